@@ -1,6 +1,7 @@
 // Fused, temporally blocked 2D kernels for the fine levels of the V-cycle
 // (Algorithm 1), constant stencil, red-black Gauss-Seidel. These scalar
-// instances run the FP64 levels; FP32 levels run the packed FP32x2 instances
+// instances run the FP64 levels of batches and those that the fixed-point
+// passes (fx2d.cuh) leave out; FP32 levels run the packed FP32x2 instances
 // of the same design (fused2d_x2.cuh, and fused2d_x2v.cuh for the variable
 // stencil).
 //

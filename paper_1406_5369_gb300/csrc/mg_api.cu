@@ -348,13 +348,38 @@ bool level_fused(mg_ctx *c, int l) {
          mg::d2::fused_ok(c->lv[l], c->lv[l + 1], fused_sweeps(c, c->opt.nu2));
 }
 
+// True when level l runs on the fixed-point 2D passes (fx2d.cuh): FP64
+// constant-stencil levels of either smoother. A tile size set by the caller
+// keeps the block-tile kernels up to it.
+bool level_fx(const mg_ctx *c, int l) {
+  const Level &L = c->lv[l];
+  return c->opt.fuse && !c->dc && l + 1 < c->nl && c->opt.nu1 >= 1 && c->opt.nu2 >= 1 &&
+         L.n > c->opt.tile_max_n && L.n > mg::coarse_top_n(c->dim, true) && c->opt.fuse_depth == 0 &&
+         c->lv[l + 1].dtype == mg::F64 && mg::d2::fx_ok(L, (int)c->opt.smoother, c->opt.omega);
+}
+
+// One fixed-point pass of level l (mg::d2::fx_pass) from the live solution buffer to the other.
+mg_status fx_pass(mg_ctx *c, int l, int kind, int nu, bool zero, bool corr, bool restr, int *nparts, cudaStream_t s) {
+  Level &L = c->lv[l], &C = c->lv[l + 1];
+  TLAUNCH(c, kind, l, s,
+          mg::d2::fx_pass(L, &C, (int)c->opt.smoother, c->opt.omega, nu, L.u[L.cur], L.u[L.cur ^ 1], zero,
+                          corr ? C.u[C.cur] : nullptr, restr ? C.f : nullptr, nparts ? c->partials : nullptr, nparts,
+                          c->opt.tile_rows, s));
+  L.cur ^= 1;
+  return MG_OK;
+}
+
 // Algorithm 1 from level l down: presmooth, residual, restrict, zero the
 // coarse solution, recurse, interpolate and correct, postsmooth. `zero`
 // says that u_l is zero on entry (every coarse level, and the finest level
 // of a defect-correction step), which lets the fused kernels skip reading it.
-mg_status vcycle_rec(mg_ctx *c, int l, bool zero, cudaStream_t s) {
+// `nparts` (finest level, may be NULL): a level whose last pass also forms
+// the residual leaves the partial sums of its square in c->partials and their
+// number here, otherwise 0.
+mg_status vcycle_rec(mg_ctx *c, int l, bool zero, cudaStream_t s, int *nparts = nullptr) {
   NvtxRange range(c->level_name[l]);
   mg_status st;
+  if (nparts) *nparts = 0;
   if (c->opt.fuse && c->dim == 2 && c->lv[l].n > mg::coarse_top_n(c->dim, !c->dc) &&
       mg::cluster_ok(c->lv, l, c->nl, (int)c->opt.smoother, !c->dc, c->opt.cluster_max_n)) {
     TLAUNCH(c, MG_KERNEL_COARSE, l, s,
@@ -371,6 +396,25 @@ mg_status vcycle_rec(mg_ctx *c, int l, bool zero, cudaStream_t s) {
     return op_coarse(c, s, MG_KERNEL_COARSE);
   }
   Level &L = c->lv[l], &C = c->lv[l + 1];
+  if (level_fx(c, l)) {
+    // passes of at most two sweeps; more of them are passes of their own
+    int left = c->opt.nu1;
+    if (zero && left > 2) {
+      if ((st = op_zero_u(c, l, s))) return st;
+      zero = false;
+    }
+    for (; left > 2; left -= 2)
+      if ((st = fx_pass(c, l, MG_KERNEL_PRESMOOTH, 2, false, false, false, nullptr, s))) return st;
+    if ((st = fx_pass(c, l, MG_KERNEL_PRESMOOTH, left, zero, false, true, nullptr, s))) return st;
+    if ((st = vcycle_rec(c, l + 1, true, s))) return st;
+    left = c->opt.nu2;
+    const int first = left > 2 ? 2 : left;
+    left -= first;
+    if ((st = fx_pass(c, l, MG_KERNEL_POSTSMOOTH, first, false, true, false, left ? nullptr : nparts, s))) return st;
+    for (; left > 0; left -= 2)
+      if ((st = fx_pass(c, l, MG_KERNEL_POSTSMOOTH, left > 2 ? 2 : left, false, false, false, nullptr, s))) return st;
+    return MG_OK;
+  }
   if (level_fused(c, l)) {
       // fuse_depth d < nu: nu - d separate sweeps before the fused pre-smoothing
     // pass and after the fused post-smoothing pass
@@ -529,7 +573,13 @@ mg_status dc_inner_and_update(mg_ctx *c, bool norm, cudaStream_t s) {
 mg_status record(mg_ctx *c, int kind, cudaStream_t s) {
   mg_status st;
   if (!c->dc) {
-    if ((st = vcycle_rec(c, 0, false, s))) return st;
+    int np = 0;
+    if ((st = vcycle_rec(c, 0, false, s, kind == 1 ? &np : nullptr))) return st;
+    if (kind == 1 && np > 0) {
+      TLAUNCH(c, MG_KERNEL_NORM, 0, s,
+              mg::norm_finalize_ex(c->partials, np, c->norm_out, nullptr, nullptr, interior_count(c->lv[0]), s));
+      return MG_OK;
+    }
     if (kind == 1) return op_norm(c, 0, s);
     return MG_OK;
   }

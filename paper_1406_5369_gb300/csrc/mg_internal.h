@@ -101,6 +101,20 @@ cudaError_t postpre_fused(const Level &L, const void *uin, void *uout, const Lev
                           int nu2, int nu1, double omega, int R, int tile_max_n, cudaStream_t s);
 }  // namespace d2
 
+// Fixed-point passes of the FP64 constant-stencil 2D levels (fx2d.cuh), for
+// both smoothers: nu (1 or 2) sweeps from u_in (or from zero) to u_out; before
+// them the correction by the coarse solution ec, after them the restricted
+// residual into fc, or the partial sums of its square (none where NULL).
+// fx_ok: the level takes them, from 65^2 on (65^2, V(2,1), pre + post: 34 us
+// against 52 us on the FP64 tile kernels; 33^2 and below are one launch of the
+// coarse cycle).
+namespace d2 {
+constexpr int kFxMinN = 65;
+bool fx_ok(const Level &L, int smoother, double omega);
+cudaError_t fx_pass(const Level &L, const Level *C, int smoother, double omega, int nu, const void *uin, void *uout,
+                    bool zero, const void *ec, void *fc, double *partials, int *nparts, int rows, cudaStream_t s);
+}  // namespace d2
+
 // Streaming 2D finest-level kernels (constant stencil). dc_step: FP64 outer
 // step of defect correction (optional update u_out = u_in + e, residual ->
 // defect d, per-warp partial sums); norm_stream: per-warp partial sums of
