@@ -20,6 +20,7 @@
 
 #include <cuda_runtime.h>
 
+#include "fx2d.cuh"
 #include "mg_cc.h"
 #include "mg_internal.h"
 
@@ -281,7 +282,7 @@ struct mg_cc_ctx {
   int nl;
   Lev lv[kMaxLev];
   double *ainv;      // coarsest grid inverse, N x N
-  double *partials;  // kNormBlocks norm partial sums
+  double *partials;  // mg::kMaxPartials norm partial sums
   double *norm_out;  // one double
   cudaStream_t s;
 };
@@ -360,7 +361,7 @@ size_t layout(mg_cc_ctx *c, char *base) {
   const int nc = c->lv[c->nl - 1].n;
   const size_t N = (size_t)nc * nc * (dim == 3 ? nc : 1);
   c->ainv = take(N * N * sizeof(double));
-  c->partials = take(kNormBlocks * sizeof(double));
+  c->partials = take(mg::kMaxPartials * sizeof(double));
   c->norm_out = take(sizeof(double));
   return align256(off);
 }
@@ -447,13 +448,17 @@ mg_status op_coarse(mg_cc_ctx *c) {
   return MG_OK;
 }
 
+mg_status norm_final(mg_cc_ctx *c, int nparts) {
+  k_norm_final<<<1, kThreads, 0, c->s>>>(c->partials, nparts, c->norm_out);
+  CCK(cudaGetLastError());
+  return MG_OK;
+}
+
 mg_status op_norm(mg_cc_ctx *c, int l) {
   Lev &L = c->lv[l];
   DIMCALL(c->p.dim, k_norm_partials, kNormBlocks, kThreads, L.u[L.cur], L.f, geo_of(L), coef_of(c, L),
           c->partials);
-  k_norm_final<<<1, kThreads, 0, c->s>>>(c->partials, kNormBlocks, c->norm_out);
-  CCK(cudaGetLastError());
-  return MG_OK;
+  return norm_final(c, kNormBlocks);
 }
 
 mg_status read_norm(mg_cc_ctx *c, double *out) {
@@ -462,16 +467,80 @@ mg_status read_norm(mg_cc_ctx *c, double *out) {
   return MG_OK;
 }
 
-// Algorithm 1 from level l down; coarse levels start from zero.
-mg_status vcycle_rec(mg_cc_ctx *c, int l) {
+// 2D levels of at least this size run on the fixed-point passes of fx2d.cuh:
+// one launch per smoothing phase in place of 6 or more.
+constexpr int kFxMinN = 64;
+
+// Level l's pass constants; false: the level keeps the kernels above.
+bool fx_args(const mg_cc_ctx *c, int l, bool corr, mg::fx2::Args &a) {
+  const Lev &L = c->lv[l];
+  if (c->p.dim != 2 || L.n < kFxMinN || l + 1 >= c->nl || c->p.nu1 < 1 || c->p.nu2 < 1) return false;
+  memset(&a, 0, sizeof a);
+  const double ih2 = (double)L.n * (double)L.n;
+  return mg::fx2::set_operator(a, c->p.c[0] * ih2, c->p.c[1] * ih2, c->p.sigma, c->p.bc == MG_CC_NEUMANN ? 1 : 3,
+                               c->p.omega, corr, c->p.smoother == MG_RBGS ? 4 : 2);
+}
+bool level_fx(const mg_cc_ctx *c, int l) {
+  mg::fx2::Args a;
+  return fx_args(c, l, true, a);
+}
+
+// One pass of level l: nu (1 or 2) sweeps from the live solution (or zero) to
+// the other buffer; before them the coarse correction (corr), after them the
+// restricted residual (restr) or the partial sums of its square (nparts).
+mg_status fx_pass(mg_cc_ctx *c, int l, int nu, bool zero, bool corr, bool restr, int *nparts) {
+  Lev &L = c->lv[l], &C = c->lv[l + 1];
+  mg::fx2::Args a;
+  if (!fx_args(c, l, corr, a)) return ccfail(MG_EINVAL, "level %d has no fixed-point pass", l);
+  a.uin = L.u[L.cur];
+  a.uout = L.u[L.cur ^ 1];
+  a.f = L.f;
+  a.ec = corr ? C.u[C.cur] : nullptr;
+  a.fc = restr ? C.f : nullptr;
+  a.partials = nparts ? c->partials : nullptr;
+  a.n = L.n;
+  a.pitch = L.pitch;
+  a.nc = C.n;
+  a.pitchc = C.pitch;
+  const int out = restr ? mg::fx2::kRestrict : nparts ? mg::fx2::kNorm : mg::fx2::kNone;
+  CCK(mg::fx2::run(a, true, c->p.smoother != MG_RBGS, 0, nu, zero, corr, out, nparts, c->s));
+  L.cur ^= 1;
+  return MG_OK;
+}
+
+// Algorithm 1 from level l down; coarse levels start from zero (`zero`: u_l
+// counts as zero whatever its buffer holds). nparts (finest level, may be
+// NULL): the number of partial sums of the squared residual that the last
+// pass left in c->partials, 0 if it left none.
+mg_status vcycle_rec(mg_cc_ctx *c, int l, bool zero = false, int *nparts = nullptr) {
   mg_status st;
+  Lev &L = c->lv[l];
+  if (nparts) *nparts = 0;
+  if (level_fx(c, l)) {
+    // passes of at most two sweeps; more of them are passes of their own
+    int left = c->p.nu1;
+    if (zero && left > 2) {
+      CCK(cudaMemsetAsync(L.u[L.cur], 0, (size_t)L.count * sizeof(double), c->s));
+      zero = false;
+    }
+    for (; left > 2; left -= 2)
+      if ((st = fx_pass(c, l, 2, false, false, false, nullptr))) return st;
+    if ((st = fx_pass(c, l, left, zero, false, true, nullptr))) return st;
+    if ((st = vcycle_rec(c, l + 1, true))) return st;
+    left = c->p.nu2;
+    const int first = left > 2 ? 2 : left;
+    left -= first;
+    if ((st = fx_pass(c, l, first, false, true, false, left ? nullptr : nparts))) return st;
+    for (; left > 0; left -= 2)
+      if ((st = fx_pass(c, l, left > 2 ? 2 : left, false, false, false, nullptr))) return st;
+    return MG_OK;
+  }
+  if (zero) CCK(cudaMemsetAsync(L.u[L.cur], 0, (size_t)L.count * sizeof(double), c->s));
   if (l == c->nl - 1) return op_coarse(c);
   if ((st = op_smooth(c, l, c->p.nu1))) return st;
   if ((st = op_residual(c, l))) return st;
   if ((st = op_restrict(c, l))) return st;
-  Lev &C = c->lv[l + 1];
-  CCK(cudaMemsetAsync(C.u[C.cur], 0, (size_t)C.count * sizeof(double), c->s));
-  if ((st = vcycle_rec(c, l + 1))) return st;
+  if ((st = vcycle_rec(c, l + 1, true))) return st;
   if ((st = op_prolong(c, l))) return st;
   return op_smooth(c, l, c->p.nu2);
 }
@@ -634,7 +703,8 @@ mg_status mg_cc_solve(mg_cc_ctx *c, double tol, int *iters, double *relres, doub
   int k = 0;
   double rho = r0 > 0.0 ? 1.0 : 0.0;
   while (r0 > 0.0 && rho > tol && k < c->p.maxit) {
-    if ((st = vcycle_rec(c, 0)) || (st = op_norm(c, 0))) return st;
+    int np = 0;
+    if ((st = vcycle_rec(c, 0, false, &np)) || (st = np ? norm_final(c, np) : op_norm(c, 0))) return st;
     double rk;
     if ((st = read_norm(c, &rk))) return st;
     rho = rk / r0;

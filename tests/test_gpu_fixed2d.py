@@ -103,3 +103,29 @@ def test_non_finite_values(bad):
     assert np.array_equal(res["edge", True], res["plain", True])
     assert np.array_equal(np.isfinite(res["hole", True]), np.isfinite(res["hole", False]))
     assert not np.isfinite(res["hole", True]).all()
+
+
+# 64: one strip and a ragged one; 512, 1024: several chunks; sigma h^2 from 1e-6 to 0.8 and zero
+@pytest.mark.parametrize("n,bc,sigma,smoother,omega,nu,c", [
+    (64, "neumann", 3000.0, "rbgs", 1.0, (2, 2), (1.0, 1.0)),
+    (128, "dirichlet", 0.0, "rbgs", 1.1, (2, 1), (1.0, 1.0)),
+    (256, "neumann", 1.0, "jacobi", 0.8, (3, 2), (1.0, 1.0)),
+    (512, "dirichlet", 50.0, "rbgs", 1.0, (1, 3), (0.8, 1.25)),
+    (512, "neumann", 10.0, "jacobi", 0.8, (2, 2), (1.25, 0.9)),
+    (1024, "neumann", 1.0, "rbgs", 1.0, (2, 2), (1.0, 1.0)),
+    (64, "neumann", 1e5, "rbgs", 1.0, (2, 2), (1.0, 1.0)),  # sigma h^2 = 24: stays on the FP64 kernels
+])
+def test_cell_cycles_match_oracle(n, bc, sigma, smoother, omega, nu, c):
+    need_gpu()
+    from paper_1406_5369_gb300 import CCSolver
+    f, u0 = synth.uniform(21, (n, n)) - 0.5, synth.uniform(22, (n, n))
+    s = CCSolver(2, n, c=c, sigma=sigma, bc=bc, smoother=smoother, omega=omega, nu1=nu[0], nu2=nu[1], maxit=3)
+    s.set_rhs(f)
+    s.set_solution(u0)
+    _, _, hist = s.solve(0.0, raise_on_noconv=False)
+    ref = oracle.CCHierarchy(2, n, c=c, sigma=sigma, bc=bc, smoother=SM[smoother], omega=omega, nu1=nu[0], nu2=nu[1])
+    ref.set_rhs(f)
+    ref.set_u(u0)
+    rho = ref.solve(0.0, 3)
+    assert np.max(np.abs(hist - rho) / np.maximum(1.0, rho)) <= 1e-12, (hist, rho)
+    assert rel_err(s.get_field(0, "u"), ref.get_u()) <= 1e-12
