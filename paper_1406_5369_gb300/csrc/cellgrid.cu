@@ -508,6 +508,32 @@ mg_status fx_pass(mg_cc_ctx *c, int l, int nu, bool zero, bool corr, bool restr,
   return MG_OK;
 }
 
+// The cluster V-cycle of levels l .. nl-1 (small2d.cuh); lg = 0 when the level does not take it.
+mg::Small2D small_desc(const mg_cc_ctx *c, int l, bool zero) {
+  mg::Small2D d;
+  memset(&d, 0, sizeof d);
+  const Lev &L = c->lv[l];
+  if (c->p.dim != 2 || L.n > (1 << mg::kSmallTopLog) || l + 1 >= c->nl) return d;
+  while ((1 << d.lg) < L.n) d.lg++;
+  const double ih2 = (double)L.n * (double)L.n;
+  d.cell = true;
+  d.nlev = c->nl - l;
+  d.kx = c->p.c[0] * ih2;
+  d.ky = c->p.c[1] * ih2;
+  d.sigma = c->p.sigma;
+  d.edge = c->p.bc == MG_CC_NEUMANN ? 1 : 3;
+  d.smoother = (int)c->p.smoother;
+  d.nu1 = c->p.nu1;
+  d.nu2 = c->p.nu2;
+  d.omega = c->p.omega;
+  d.zero = zero;
+  d.f = L.f;
+  d.u = L.u[L.cur];
+  d.pitch = L.pitch;
+  d.dense = c->ainv;
+  return d;
+}
+
 // Algorithm 1 from level l down; coarse levels start from zero (`zero`: u_l
 // counts as zero whatever its buffer holds). nparts (finest level, may be
 // NULL): the number of partial sums of the squared residual that the last
@@ -516,6 +542,14 @@ mg_status vcycle_rec(mg_cc_ctx *c, int l, bool zero = false, int *nparts = nullp
   mg_status st;
   Lev &L = c->lv[l];
   if (nparts) *nparts = 0;
+  {
+    mg::Small2D d = small_desc(c, l, zero);
+    if (d.lg > 0 && mg::small2d_ok(d)) {
+      if (nparts) d.partials = c->partials;
+      CCK(mg::small2d_cycle(d, nparts, c->s));
+      return MG_OK;
+    }
+  }
   if (level_fx(c, l)) {
     // passes of at most two sweeps; more of them are passes of their own
     int left = c->p.nu1;
@@ -591,6 +625,7 @@ mg_status mg_cc_create(const mg_cc_params *p, void *arena, size_t arena_bytes, m
   if (!c) return ccfail(MG_ENOMEM, "host allocation of the context failed");
   c->p = *p;
   c->s = (cudaStream_t)p->stream;
+  if (p->dim == 2) mg::small2d_probe();
   size_t need = layout(c, nullptr);
   if (arena_bytes < need) {
     free(c);

@@ -358,6 +358,31 @@ bool level_fx(const mg_ctx *c, int l) {
          c->lv[l + 1].dtype == mg::F64 && mg::d2::fx_ok(L, (int)c->opt.smoother, c->opt.omega);
 }
 
+// The cluster V-cycle of levels l .. nl-1 (small2d.cuh); lg = 0 when the
+// context or the level does not take it. cluster_max_n sets its largest level.
+mg::Small2D small_desc(const mg_ctx *c, int l, bool zero) {
+  mg::Small2D d;
+  memset(&d, 0, sizeof d);
+  const Level &L = c->lv[l];
+  const int top = c->opt.cluster_max_n > 0 ? c->opt.cluster_max_n : (1 << mg::kSmallTopLog) + 1;
+  if (!c->opt.fuse || c->dc || c->dim != 2 || c->variable || L.n > top || l + 1 >= c->nl) return d;
+  while ((1 << d.lg) + 1 < L.n) d.lg++;
+  d.nlev = c->nl - l;
+  d.kx = L.c[0] * L.inv_h2;
+  d.ky = L.c[1] * L.inv_h2;
+  d.edge = 2;
+  d.smoother = (int)c->opt.smoother;
+  d.nu1 = c->opt.nu1;
+  d.nu2 = c->opt.nu2;
+  d.omega = c->opt.omega;
+  d.zero = zero;
+  d.f = (const double *)L.f;
+  d.u = (double *)L.u[L.cur];
+  d.pitch = L.pitch;
+  d.dense = c->lv[c->nl - 1].dense;
+  return d;
+}
+
 // One fixed-point pass of level l (mg::d2::fx_pass) from the live solution buffer to the other.
 mg_status fx_pass(mg_ctx *c, int l, int kind, int nu, bool zero, bool corr, bool restr, int *nparts, cudaStream_t s) {
   Level &L = c->lv[l], &C = c->lv[l + 1];
@@ -380,6 +405,14 @@ mg_status vcycle_rec(mg_ctx *c, int l, bool zero, cudaStream_t s, int *nparts = 
   NvtxRange range(c->level_name[l]);
   mg_status st;
   if (nparts) *nparts = 0;
+  {
+    mg::Small2D d = small_desc(c, l, zero);
+    if (d.lg > 0 && mg::small2d_ok(d)) {
+      if (nparts) d.partials = c->partials;
+      TLAUNCH(c, MG_KERNEL_COARSE, l, s, mg::small2d_cycle(d, nparts, s));
+      return MG_OK;
+    }
+  }
   if (c->opt.fuse && c->dim == 2 && c->lv[l].n > mg::coarse_top_n(c->dim, !c->dc) &&
       mg::cluster_ok(c->lv, l, c->nl, (int)c->opt.smoother, !c->dc, c->opt.cluster_max_n)) {
     TLAUNCH(c, MG_KERNEL_COARSE, l, s,
@@ -766,6 +799,7 @@ mg_status mg_create(int dim, int n, const mg_const_stencil *stencil, const doubl
   c->capturing_slot = -1;
   // the device check of the cluster cycle runs here, never inside a capture
   if (dim == 2 && c->dc && opt->fuse && opt->smoother == MG_RBGS) mg::cluster_probe();
+  if (dim == 2 && !c->dc && opt->fuse) mg::small2d_probe();
   for (int d = 0; d < 3; d++) c->lv[0].c[d] = c3[d];
   size_t need = layout(c, nullptr);
   if (arena_bytes < need) {

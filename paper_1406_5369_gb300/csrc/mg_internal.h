@@ -205,6 +205,30 @@ void coarse_args_set_live(void *args, const int *live);
 cudaError_t coarse_cycle_batched(const void *list_dev, int count, int dim, bool var, bool fp64, size_t smem,
                                  cudaStream_t s);
 
+// FP64 V-cycle of the small 2D levels on one thread-block cluster
+// (small2d.cuh): node-based or cell-centred constant-stencil grids, either
+// smoother. The top level has 2^lg cells per dimension, nlev levels down to
+// the coarsest. small2d_probe asks the device once whether the cluster fits
+// (outside any stream capture); small2d_ok answers no until it has run.
+struct Small2D {
+  bool cell;
+  int lg, nlev;
+  double kx, ky, sigma;  // axis coefficients over h^2 and reaction term of the top level
+  int edge;              // weight of u on an axis with a boundary face: 2 (node), 1 (zero flux), 3 (fixed value)
+  int smoother, nu1, nu2;
+  double omega;
+  bool zero;             // start from u = 0
+  const double *f;
+  double *u;
+  int pitch;
+  const double *dense;   // coarsest inverse, NULL for a single node
+  double *partials;      // sums of the squared residual of the result, one per block (NULL: none)
+};
+constexpr int kSmallTopLog = 7;  // largest level taken by default
+void small2d_probe();
+bool small2d_ok(const Small2D &d);
+cudaError_t small2d_cycle(const Small2D &d, int *nparts, cudaStream_t s);
+
 // Sets the message mg_last_error() returns on the calling thread.
 void set_error_message(const char *msg);
 

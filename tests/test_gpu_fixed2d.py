@@ -129,3 +129,64 @@ def test_cell_cycles_match_oracle(n, bc, sigma, smoother, omega, nu, c):
     rho = ref.solve(0.0, 3)
     assert np.max(np.abs(hist - rho) / np.maximum(1.0, rho)) <= 1e-12, (hist, rho)
     assert rel_err(s.get_field(0, "u"), ref.get_u()) <= 1e-12
+
+
+# every depth of the cluster cycle, up to its largest level (257), alone and below the streaming passes
+@pytest.mark.parametrize("n,smoother,omega,nu,c,nc,top", [
+    (5, "rbgs", 1.0, (2, 1), (1.0, 1.0), 3, 0),
+    (9, "jacobi", 0.8, (1, 2), (1.0, 2.0), 5, 0),
+    (17, "rbgs", 1.2, (0, 2), (1.0, 1.0), 9, 0),
+    (33, "jacobi", 0.7, (2, 1), (1.0, 1.0), 3, 0),
+    (65, "rbgs", 1.0, (2, 0), (1.5, 0.5), 3, 0),
+    (65, "jacobi", 0.8, (3, 2), (1.0, 1.0), 9, 0),
+    (129, "rbgs", 1.0, (2, 1), (1.0, 1.0), 3, 0),
+    (129, "jacobi", 0.8, (1, 1), (1.0, 1.0), 5, 0),
+    (257, "rbgs", 1.1, (2, 2), (1.0, 1.0), 9, 257),
+    (513, "jacobi", 0.8, (1, 2), (1.0, 1.0), 3, 0),
+])
+def test_cluster_cycle_matches_oracle(n, smoother, omega, nu, c, nc, top):
+    f = synth.uniform_rhs(2, n, 31)
+    b = synth.uniform(32, (n, n)) * 0.1
+    s = solver(n, smoother=smoother, omega=omega, nu1=nu[0], nu2=nu[1], stencil=c + (1.0,), maxit=3, dirichlet=b,
+               coarsest_n=nc, cluster_max_n=top)
+    s.set_rhs(f)
+    _, _, hist = s.solve(0.0, raise_on_noconv=False)
+    ref = oracle.Hierarchy(2, n, c=c, smoother=SM[smoother], omega=omega, nu1=nu[0], nu2=nu[1], coarsest_n=nc)
+    u0 = np.array(b)
+    u0[1:-1, 1:-1] = 0.0
+    ref.set_u(u0)
+    ref.set_rhs(f)
+    rho = ref.solve(0.0, 3)
+    assert np.max(np.abs(hist - rho) / np.maximum(1.0, rho)) <= 1e-12, (hist, rho)
+    u = s.get_solution()
+    assert rel_err(u, ref.get_u()) <= 1e-12
+    assert np.array_equal(u[0], b[0]) and np.array_equal(u[:, -1], b[:, -1])
+
+
+@pytest.mark.parametrize("n,bc,sigma,smoother,omega,nu,nc", [
+    (2, "dirichlet", 0.0, "rbgs", 1.0, (2, 1), 1),
+    (4, "neumann", 5.0, "jacobi", 0.8, (1, 2), 1),
+    (8, "dirichlet", 1.0, "rbgs", 1.2, (0, 2), 4),
+    (32, "neumann", 100.0, "rbgs", 1.0, (2, 2), 2),
+    (64, "neumann", 1.0, "jacobi", 0.8, (3, 2), 1),
+    (64, "dirichlet", 2000.0, "rbgs", 1.0, (1, 0), 4),
+    (128, "dirichlet", 0.0, "jacobi", 0.8, (1, 2), 2),
+    (128, "neumann", 0.01, "rbgs", 1.0, (2, 2), 1),
+])
+def test_cell_cluster_cycle_matches_oracle(n, bc, sigma, smoother, omega, nu, nc):
+    need_gpu()
+    from paper_1406_5369_gb300 import CCSolver
+    c = (1.0, 0.7)
+    f, u0 = synth.uniform(21, (n, n)) - 0.5, synth.uniform(22, (n, n))
+    s = CCSolver(2, n, c=c, sigma=sigma, bc=bc, smoother=smoother, omega=omega, nu1=nu[0], nu2=nu[1], maxit=3,
+                 coarsest_n=nc)
+    s.set_rhs(f)
+    s.set_solution(u0)
+    _, _, hist = s.solve(0.0, raise_on_noconv=False)
+    ref = oracle.CCHierarchy(2, n, c=c, sigma=sigma, bc=bc, smoother=SM[smoother], omega=omega, nu1=nu[0],
+                             nu2=nu[1], coarsest_n=nc)
+    ref.set_rhs(f)
+    ref.set_u(u0)
+    rho = ref.solve(0.0, 3)
+    assert np.max(np.abs(hist - rho) / np.maximum(1.0, rho)) <= 1e-12, (hist, rho)
+    assert rel_err(s.get_field(0, "u"), ref.get_u()) <= 1e-12
