@@ -1,9 +1,9 @@
 // Implicit Euler steps of nonlinear complex diffusion (include/mg_cd.h):
 // Sec. 4's second test problem on cell-centred grids, complex FP64.
 //
-// Layout: level l has n_l = n / 2^l cells per dimension and seven complex
+// Layout: level l has n_l = n / 2^l cells per dimension and eight complex
 // fields (double2: real, imaginary) u[0], u[1] (Jacobi ping-pong), f, r, the
-// face coefficients gx, gy and wd = omega / diag per cell, rows padded to 128
+// face coefficients gx, gy, wd = omega / diag and gf = wd f per cell, rows padded to 128
 // bytes (pitch = n_l rounded up to 8 complex values), x fastest, no ghost
 // cells. One thread per cell (per cell of the swept colour for red-black
 // Gauss-Seidel), rows on blockIdx.y. The arithmetic is FP64 throughout and
@@ -73,43 +73,6 @@ __device__ __forceinline__ double2 apply(const double2 *__restrict__ u, const do
   }
   diag = make_double2(1.0 + s * gs.x, s * gs.y);
   return cadd(u0, cscale(s, acc));
-}
-
-// Cell diffusivity g(Im u) = e^{i theta} w, w = 1 / (1 + (Im u / (kappa theta))^2).
-__device__ __forceinline__ double2 diffusivity(double2 u, double er, double ei, double inv_kt) {
-  const double t = u.y * inv_kt;
-  const double w = 1.0 / (1.0 + t * t);
-  return make_double2(er * w, ei * w);
-}
-
-__global__ void k_faces(const double2 *__restrict__ u, double2 *__restrict__ gx, double2 *__restrict__ gy, Geo g,
-                        double er, double ei, double inv_kt) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-  if (i >= g.n) return;
-  const long long p = (long long)j * g.sy + i;
-  const double2 gp = diffusivity(u[p], er, ei, inv_kt);
-  double2 fx = make_double2(0.0, 0.0), fy = make_double2(0.0, 0.0);
-  if (i + 1 < g.n) fx = cscale(0.5, cadd(gp, diffusivity(u[p + 1], er, ei, inv_kt)));
-  if (j + 1 < g.n) fy = cscale(0.5, cadd(gp, diffusivity(u[p + g.sy], er, ei, inv_kt)));
-  gx[p] = fx;
-  gy[p] = fy;
-}
-
-// Coarse x-face (I, J) | (I+1, J): mean of the fine faces at x index 2I+1,
-// rows 2J and 2J+1; coarse y-face (I, J) | (I, J+1): mean of the fine faces
-// at row 2J+1, columns 2I and 2I+1.
-__global__ void k_coarsen_faces(const double2 *__restrict__ gxf, const double2 *__restrict__ gyf, Geo gf,
-                                double2 *__restrict__ gxc, double2 *__restrict__ gyc, Geo gc) {
-  const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y;
-  if (I >= gc.n) return;
-  const long long P = (long long)J * gc.sy + I;
-  double2 fx = make_double2(0.0, 0.0), fy = make_double2(0.0, 0.0);
-  if (I + 1 < gc.n)
-    fx = cscale(0.5, cadd(gxf[(long long)(2 * J) * gf.sy + 2 * I + 1], gxf[(long long)(2 * J + 1) * gf.sy + 2 * I + 1]));
-  if (J + 1 < gc.n)
-    fy = cscale(0.5, cadd(gyf[(long long)(2 * J + 1) * gf.sy + 2 * I], gyf[(long long)(2 * J + 1) * gf.sy + 2 * I + 1]));
-  gxc[P] = fx;
-  gyc[P] = fy;
 }
 
 // omega / diag_p of every cell (diag as in apply).
@@ -215,10 +178,195 @@ __global__ void k_norm_final(const double *__restrict__ partials, int count, dou
   if (threadIdx.x == 0) out[0] = sqrt(a);
 }
 
+// ------------------------------------------------------------------------
+// Kernels for faces that share one phase. Every face coefficient of a step is
+// g = e^{i theta} w with a real w in (0, 1] (means of real weights stay so on
+// the coarse levels), and FP64 instructions are what the passes are bound by
+// (one per cell and pass of 2048^2 takes 7 us; the memory of a whole sweep
+// 50 us). So the sums over the four faces are formed with the real weights,
+// two FP64 instructions per face instead of four or more, and the phase is
+// applied once, inside a coefficient of the cell:
+//   smoother  u' = (1 - omega) u + g + q sum_f w_f u_q,   g = wd f, q = wd s e^{i theta}
+//             (14 FP64 instructions per cell, 42 with complex faces), and
+//             u' = g on the first sweep from zero;
+//   residual  r = f - u - s e^{i theta} sum_f w_f (u_p - u_q);
+//   its mean over a coarse cell's four cells needs the eight outer faces only,
+//             since what crosses an inner face cancels (13 per cell, was 40).
+// w[p] = (face p | p + 1, face p | row below); both are zero across the edge.
+struct Ph {
+  double x, y;  // s e^{i theta}
+};
+
+__device__ __forceinline__ void face_add(double2 &a, double w, double2 v) {
+  a.x = fma(w, v.x, a.x);
+  a.y = fma(w, v.y, a.y);
+}
+__device__ __forceinline__ double2 cfma(double2 a, double2 b, double2 c) {  // c + a b
+  return make_double2(fma(-a.y, b.y, fma(a.x, b.x, c.x)), fma(a.y, b.x, fma(a.x, b.y, c.y)));
+}
+
+constexpr int kBX = 32, kBY = 8;  // block of the kernels below
+__device__ __forceinline__ bool cell(int n, int &i, int &j) {
+  i = blockIdx.x * kBX + threadIdx.x;
+  j = blockIdx.y * kBY + threadIdx.y;
+  return i < n && j < n;
+}
+
+// sum_f w_f u_q
+__device__ __forceinline__ double2 face_sum(const double2 *__restrict__ u, const double2 *__restrict__ w, long long p,
+                                            int i, int j, const Geo &g) {
+  const double2 wp = w[p];
+  double2 a = make_double2(0.0, 0.0);
+  if (i + 1 < g.n) face_add(a, wp.x, u[p + 1]);
+  if (i > 0) face_add(a, w[p - 1].x, u[p - 1]);
+  if (j + 1 < g.n) face_add(a, wp.y, u[p + g.sy]);
+  if (j > 0) face_add(a, w[p - g.sy].y, u[p - g.sy]);
+  return a;
+}
+
+__global__ void __launch_bounds__(kBX * kBY) kr_jacobi(const double2 *__restrict__ uin, double2 *__restrict__ uout,
+                                                       const double2 *__restrict__ gf, const double2 *__restrict__ q,
+                                                       const double2 *__restrict__ w, Geo g, double gamma) {
+  int i, j;
+  if (!cell(g.n, i, j)) return;
+  const long long p = (long long)j * g.sy + i;
+  double2 v = cfma(q[p], face_sum(uin, w, p, i, j, g), gf[p]);
+  if (gamma != 0.0) face_add(v, gamma, uin[p]);
+  uout[p] = v;
+}
+
+__global__ void __launch_bounds__(kBX * kBY) kr_rbgs_half(double2 *u, const double2 *__restrict__ gf,
+                                                          const double2 *__restrict__ q,
+                                                          const double2 *__restrict__ w, Geo g, double gamma,
+                                                          int color) {
+  const int j = blockIdx.y * kBY + threadIdx.y;
+  const int i = 2 * (blockIdx.x * kBX + threadIdx.x) + ((color + j) & 1);
+  if (i >= g.n || j >= g.n) return;
+  const long long p = (long long)j * g.sy + i;
+  double2 v = cfma(q[p], face_sum(u, w, p, i, j, g), gf[p]);
+  if (gamma != 0.0) face_add(v, gamma, u[p]);
+  u[p] = v;
+}
+
+// Coarse cell (I, J): f = mean of the four residuals, g = wd f, and u after the
+// first sweep (Jacobi: g) or red half-sweep from zero; u = 0 when there is no
+// pre-smoothing (first = 0: none, 1: Jacobi, 2: red-black).
+__global__ void __launch_bounds__(kBX * kBY)
+    kr_restrict(const double2 *__restrict__ u, const double2 *__restrict__ f, const double2 *__restrict__ w, Geo g,
+                Ph ph, double2 *__restrict__ fc, double2 *__restrict__ gfc, double2 *__restrict__ uc,
+                const double2 *__restrict__ wdc, Geo gc, int first) {
+  int I, J;
+  if (!cell(gc.n, I, J)) return;
+  const int i = 2 * I, j = 2 * J;
+  const long long p = (long long)j * g.sy + i, sy = g.sy;
+  const double2 a = u[p], b = u[p + 1], c = u[p + sy], d = u[p + sy + 1];
+  double2 s = make_double2(0.0, 0.0);
+  if (i > 0) {
+    face_add(s, w[p - 1].x, csub(a, u[p - 1]));
+    face_add(s, w[p + sy - 1].x, csub(c, u[p + sy - 1]));
+  }
+  if (i + 2 < g.n) {
+    face_add(s, w[p + 1].x, csub(b, u[p + 2]));
+    face_add(s, w[p + sy + 1].x, csub(d, u[p + sy + 2]));
+  }
+  if (j > 0) {
+    face_add(s, w[p - sy].y, csub(a, u[p - sy]));
+    face_add(s, w[p - sy + 1].y, csub(b, u[p - sy + 1]));
+  }
+  if (j + 2 < g.n) {
+    face_add(s, w[p + sy].y, csub(c, u[p + 2 * sy]));
+    face_add(s, w[p + sy + 1].y, csub(d, u[p + 2 * sy + 1]));
+  }
+  double2 r = cadd(cadd(csub(f[p], a), csub(f[p + 1], b)), cadd(csub(f[p + sy], c), csub(f[p + sy + 1], d)));
+  r = cscale(0.25, cfma(make_double2(-ph.x, -ph.y), s, r));
+  const long long P = (long long)J * gc.sy + I;
+  const double2 v = cmul(wdc[P], r);
+  fc[P] = r;
+  gfc[P] = v;
+  uc[P] = first == 1 || (first == 2 && ((I + J) & 1) == 0) ? v : make_double2(0.0, 0.0);
+}
+
+// Cell diffusivity g(Im u) = e^{i theta} w, w = 1 / (1 + (Im u / (kappa theta))^2): the
+// weight, one division per cell.
+__global__ void __launch_bounds__(kBX * kBY) kr_weight(const double2 *__restrict__ u, double *__restrict__ wc, Geo g,
+                                                       double inv_kt) {
+  int i, j;
+  if (!cell(g.n, i, j)) return;
+  const long long p = (long long)j * g.sy + i;
+  const double t = u[p].y * inv_kt;
+  wc[p] = 1.0 / (1.0 + t * t);
+}
+// Fine face weights: means of the two cells'. Coarse x-face (I, J) | (I+1, J):
+// mean of the fine faces at x index 2I+1, rows 2J and 2J+1; coarse y-face
+// (I, J) | (I, J+1): mean of the fine faces at row 2J+1, columns 2I and 2I+1.
+__global__ void __launch_bounds__(kBX * kBY) kr_faces(const double *__restrict__ wc, double2 *__restrict__ w, Geo g) {
+  int i, j;
+  if (!cell(g.n, i, j)) return;
+  const long long p = (long long)j * g.sy + i;
+  const double a = wc[p];
+  w[p] = make_double2(i + 1 < g.n ? 0.5 * (a + wc[p + 1]) : 0.0, j + 1 < g.n ? 0.5 * (a + wc[p + g.sy]) : 0.0);
+}
+__global__ void __launch_bounds__(kBX * kBY) kr_coarsen_faces(const double2 *__restrict__ wf, Geo gf,
+                                                              double2 *__restrict__ wc, Geo gc) {
+  int I, J;
+  if (!cell(gc.n, I, J)) return;
+  const long long p = (long long)(2 * J) * gf.sy + 2 * I, sy = gf.sy;
+  wc[(long long)J * gc.sy + I] = make_double2(I + 1 < gc.n ? 0.5 * (wf[p + 1].x + wf[p + sy + 1].x) : 0.0,
+                                              J + 1 < gc.n ? 0.5 * (wf[p + sy].y + wf[p + sy + 1].y) : 0.0);
+}
+// wd = omega / diag, q = wd s e^{i theta}; with f also g = wd f (the finest level).
+__global__ void __launch_bounds__(kBX * kBY) kr_diag(const double2 *__restrict__ w, Geo g, Ph ph, double omega,
+                                                     double2 *__restrict__ wd, double2 *__restrict__ q,
+                                                     const double2 *__restrict__ f, double2 *__restrict__ gf) {
+  int i, j;
+  if (!cell(g.n, i, j)) return;
+  const long long p = (long long)j * g.sy + i;
+  double s = w[p].x + w[p].y;
+  if (i > 0) s += w[p - 1].x;
+  if (j > 0) s += w[p - g.sy].y;
+  const double2 d = cdiv(make_double2(omega, 0.0), make_double2(fma(ph.x, s, 1.0), ph.y * s));
+  wd[p] = d;
+  q[p] = cmul(d, make_double2(ph.x, ph.y));
+  if (f) gf[p] = cmul(d, f[p]);
+}
+// The complex faces from the weights, in place: gx holds w on entry.
+__global__ void __launch_bounds__(kBX * kBY) kr_expand(double2 *gx, double2 *__restrict__ gy, Geo g, double er,
+                                                       double ei) {
+  int i, j;
+  if (!cell(g.n, i, j)) return;
+  const long long p = (long long)j * g.sy + i;
+  const double2 w = gx[p];
+  gx[p] = make_double2(er * w.x, ei * w.x);
+  gy[p] = make_double2(er * w.y, ei * w.y);
+}
+
+// Norm partial sums in the order of k_norm_partials.
+__global__ void __launch_bounds__(kThreads) kr_norm_partials(const double2 *__restrict__ u, const double2 *__restrict__ f,
+                                                             const double2 *__restrict__ w, Geo g, Ph ph,
+                                                             double *__restrict__ partials) {
+  double acc = 0.0;
+  for (int j = blockIdx.x; j < g.n; j += gridDim.x)
+    for (int i = threadIdx.x; i < g.n; i += blockDim.x) {
+      const long long p = (long long)j * g.sy + i;
+      const double2 a = u[p], wp = w[p];
+      double2 s = make_double2(0.0, 0.0);
+      if (i + 1 < g.n) face_add(s, wp.x, csub(a, u[p + 1]));
+      if (i > 0) face_add(s, w[p - 1].x, csub(a, u[p - 1]));
+      if (j + 1 < g.n) face_add(s, wp.y, csub(a, u[p + g.sy]));
+      if (j > 0) face_add(s, w[p - g.sy].y, csub(a, u[p - g.sy]));
+      const double2 r = cfma(make_double2(-ph.x, -ph.y), s, csub(f[p], a));
+      acc = fma(r.x, r.x, fma(r.y, r.y, acc));
+    }
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) partials[blockIdx.x] = acc;
+}
+
+// Faces: general complex coefficients in gx, gy, or (phased, see the context)
+// real weights in gx and the smoother's q in gy.
 struct Lev {
   int n, pitch;
   long long count;
-  double2 *u[2], *f, *r, *gx, *gy, *wd;
+  double2 *u[2], *f, *r, *gx, *gy, *wd, *gf;
   int cur;
 };
 
@@ -233,6 +381,10 @@ struct mg_cd_ctx {
   Lev lv[kMaxLev];
   double *partials, *norm_out;
   cudaStream_t s;
+  // The faces are e^{i theta} times real weights (set by begin_step): V-cycles
+  // run on the kr_ kernels. A call that sets or reads faces, sets f or works on
+  // one level first expands the faces (to_complex).
+  bool phased;
 };
 
 namespace {
@@ -294,6 +446,7 @@ size_t layout(mg_cd_ctx *c, char *base) {
     L.gx = (double2 *)take(bytes);
     L.gy = (double2 *)take(bytes);
     L.wd = (double2 *)take(bytes);
+    L.gf = (double2 *)take(bytes);
     if (n == 1) break;
   }
   c->partials = (double *)take(kNormBlocks * sizeof(double));
@@ -352,10 +505,18 @@ mg_status op_coarse(mg_cd_ctx *c) {
   return MG_OK;
 }
 
+Ph phase_of(const mg_cd_ctx *c, const Lev &L) {
+  const double s = s_of(c, L);
+  return Ph{s * cos(c->p.theta), s * sin(c->p.theta)};
+}
+
 mg_status op_norm(mg_cd_ctx *c, int l) {
   Lev &L = c->lv[l];
-  k_norm_partials<<<kNormBlocks, kThreads, 0, c->s>>>(L.u[L.cur], L.f, L.gx, L.gy, geo_of(L), s_of(c, L),
-                                                       c->partials);
+  if (c->phased)
+    kr_norm_partials<<<kNormBlocks, kThreads, 0, c->s>>>(L.u[L.cur], L.f, L.gx, geo_of(L), phase_of(c, L), c->partials);
+  else
+    k_norm_partials<<<kNormBlocks, kThreads, 0, c->s>>>(L.u[L.cur], L.f, L.gx, L.gy, geo_of(L), s_of(c, L),
+                                                         c->partials);
   CDK(cudaGetLastError());
   k_norm_final<<<1, kThreads, 0, c->s>>>(c->partials, kNormBlocks, c->norm_out);
   CDK(cudaGetLastError());
@@ -368,7 +529,59 @@ mg_status read_norm(mg_cd_ctx *c, double *out) {
   return MG_OK;
 }
 
+const dim3 kBlock(kBX, kBY);
+dim3 tiles(int nx, int ny) { return dim3((unsigned)((nx + kBX - 1) / kBX), (unsigned)((ny + kBY - 1) / kBY)); }
+
+#define LAUNCH2(kern, nx, ny, ...)                                 \
+  do {                                                             \
+    kern<<<tiles((nx), (ny)), kBlock, 0, c->s>>>(__VA_ARGS__);     \
+    CDK(cudaGetLastError());                                       \
+  } while (0)
+
+// Phased faces back to complex ones on every level.
+mg_status to_complex(mg_cd_ctx *c) {
+  if (!c->phased) return MG_OK;
+  for (int l = 0; l < c->nl; l++) {
+    Lev &L = c->lv[l];
+    LAUNCH2(kr_expand, L.n, L.n, L.gx, L.gy, geo_of(L), cos(c->p.theta), sin(c->p.theta));
+  }
+  c->phased = false;
+  return MG_OK;
+}
+
+// Sweeps of level l with phased faces; skip: the first sweep (Jacobi) or red
+// half-sweep is already in u.
+mg_status phased_smooth(mg_cd_ctx *c, int l, int sweeps, bool skip) {
+  Lev &L = c->lv[l];
+  const Geo g = geo_of(L);
+  const double gamma = 1.0 - c->p.omega;
+  if (c->p.smoother == MG_RBGS) {
+    for (int h = skip ? 1 : 0; h < 2 * sweeps; h++)
+      LAUNCH2(kr_rbgs_half, (L.n + 1) / 2, L.n, L.u[L.cur], L.gf, L.gy, L.gx, g, gamma, h & 1);
+  } else {
+    for (int h = skip ? 1 : 0; h < sweeps; h++) {
+      LAUNCH2(kr_jacobi, L.n, L.n, L.u[L.cur], L.u[L.cur ^ 1], L.gf, L.gy, L.gx, g, gamma);
+      L.cur ^= 1;
+    }
+  }
+  return MG_OK;
+}
+
+// Algorithm 1 with phased faces; `begun`: u holds the first (half-)sweep from zero.
+mg_status phased_cycle(mg_cd_ctx *c, int l, bool begun) {
+  mg_status st;
+  if (l == c->nl - 1) return op_coarse(c);
+  Lev &L = c->lv[l], &C = c->lv[l + 1];
+  if ((st = phased_smooth(c, l, c->p.nu1, begun && c->p.nu1 > 0))) return st;
+  LAUNCH2(kr_restrict, C.n, C.n, L.u[L.cur], L.f, L.gx, geo_of(L), phase_of(c, L), C.f, C.gf, C.u[C.cur], C.wd,
+          geo_of(C), c->p.nu1 == 0 ? 0 : c->p.smoother == MG_RBGS ? 2 : 1);
+  if ((st = phased_cycle(c, l + 1, true))) return st;
+  if ((st = op_prolong(c, l))) return st;
+  return phased_smooth(c, l, c->p.nu2, false);
+}
+
 mg_status vcycle_rec(mg_cd_ctx *c, int l) {
+  if (c->phased) return phased_cycle(c, l, false);
   mg_status st;
   if (l == c->nl - 1) return op_coarse(c);
   if ((st = op_smooth(c, l, c->p.nu1))) return st;
@@ -481,6 +694,7 @@ mg_status mg_cd_set_field(mg_cd_ctx *c, int level, int field, const double *src)
   if (!src) return cdfail(MG_EINVAL, "src is NULL");
   double2 *dst = field_ptr(c->lv[level], field);
   if (!dst) return cdfail(MG_EINVAL, "unknown field %d", field);
+  if (field != MG_CD_U && field != MG_CD_R && (st = to_complex(c))) return st;
   if ((st = copy_in(c, c->lv[level], dst, src))) return st;
   return (field == MG_CD_GX || field == MG_CD_GY) ? op_wdiag(c, level) : MG_OK;
 }
@@ -492,6 +706,7 @@ mg_status mg_cd_get_field(mg_cd_ctx *c, int level, int field, double *dst) {
   Lev &L = c->lv[level];
   const double2 *src = field_ptr(L, field);
   if (!src) return cdfail(MG_EINVAL, "unknown field %d", field);
+  if ((field == MG_CD_GX || field == MG_CD_GY) && (st = to_complex(c))) return st;
   CDK(cudaMemcpy2DAsync(dst, (size_t)L.n * 16, src, (size_t)L.pitch * 16, (size_t)L.n * 16, (size_t)L.n,
                         cudaMemcpyDefault, c->s));
   CDK(cudaStreamSynchronize(c->s));
@@ -505,14 +720,18 @@ mg_status mg_cd_begin_step(mg_cd_ctx *c, const double *un) {
   L.cur = 0;
   if ((st = copy_in(c, L, L.f, un))) return st;
   CDK(cudaMemcpyAsync(L.u[0], L.f, (size_t)L.count * sizeof(double2), cudaMemcpyDeviceToDevice, c->s));
-  LAUNCH(k_faces, grid_of(L, L.n), L.f, L.gx, L.gy, geo_of(L), cos(c->p.theta), sin(c->p.theta),
-         1.0 / (c->p.kappa * c->p.theta));
+  double *wc = (double *)L.gy;  // q comes there last
+  LAUNCH2(kr_weight, L.n, L.n, L.f, wc, geo_of(L), 1.0 / (c->p.kappa * c->p.theta));
+  LAUNCH2(kr_faces, L.n, L.n, wc, L.gx, geo_of(L));
   for (int l = 1; l < c->nl; l++) {
     Lev &F = c->lv[l - 1], &C = c->lv[l];
-    LAUNCH(k_coarsen_faces, grid_of(C, C.n), F.gx, F.gy, geo_of(F), C.gx, C.gy, geo_of(C));
+    LAUNCH2(kr_coarsen_faces, C.n, C.n, F.gx, geo_of(F), C.gx, geo_of(C));
   }
-  for (int l = 0; l < c->nl; l++)
-    if ((st = op_wdiag(c, l))) return st;
+  for (int l = 0; l < c->nl; l++) {
+    Lev &F = c->lv[l];
+    LAUNCH2(kr_diag, F.n, F.n, F.gx, geo_of(F), phase_of(c, F), c->p.omega, F.wd, F.gy, l == 0 ? F.f : nullptr, F.gf);
+  }
+  c->phased = true;
   return MG_OK;
 }
 
@@ -520,22 +739,23 @@ mg_status mg_cd_smooth(mg_cd_ctx *c, int level, int sweeps) {
   mg_status st = level_ok(c, level, false);
   if (st) return st;
   if (sweeps < 0) return cdfail(MG_EINVAL, "sweeps must be >= 0");
+  if ((st = to_complex(c))) return st;
   return op_smooth(c, level, sweeps);
 }
 
 mg_status mg_cd_residual(mg_cd_ctx *c, int level) {
   mg_status st = level_ok(c, level, false);
-  return st ? st : op_residual(c, level);
+  return st || (st = to_complex(c)) ? st : op_residual(c, level);
 }
 
 mg_status mg_cd_restrict(mg_cd_ctx *c, int level) {
   mg_status st = level_ok(c, level, true);
-  return st ? st : op_restrict(c, level);
+  return st || (st = to_complex(c)) ? st : op_restrict(c, level);
 }
 
 mg_status mg_cd_prolongate(mg_cd_ctx *c, int level) {
   mg_status st = level_ok(c, level, true);
-  return st ? st : op_prolong(c, level);
+  return st || (st = to_complex(c)) ? st : op_prolong(c, level);
 }
 
 mg_status mg_cd_coarse_solve(mg_cd_ctx *c) {
@@ -552,6 +772,7 @@ mg_status mg_cd_residual_norm(mg_cd_ctx *c, int level, double *out) {
   mg_status st = level_ok(c, level, false);
   if (st) return st;
   if (!out) return cdfail(MG_EINVAL, "out is NULL");
+  if (level != 0 && (st = to_complex(c))) return st;
   if ((st = op_norm(c, level))) return st;
   return read_norm(c, out);
 }
