@@ -49,6 +49,7 @@ struct Coef {
   double k[3];        // c_d / h^2 = c_d n^2 (exact scaling: n is a power of two)
   double sigma, ih2;  // ih2 = 1/h^2 = n^2
   int neumann;        // ghost value u_p (Neumann) or -u_p (Dirichlet)
+  int equal;          // the k[d] are the same
   double wd[27];      // omega / diag by boundary class a_0 + 3 a_1 + 9 a_2
 };
 
@@ -191,6 +192,108 @@ template <int DIM> __device__ __forceinline__ void coarse_cell(int t, int n, int
   i = t % n;
   j = DIM == 3 ? (t / n) % n : t / n;
   k = DIM == 3 ? t / (n * n) : 0;
+}
+
+// ------------------------------------------------------------------------
+// Kernels of the V-cycle on levels that neither fx2d.cuh nor small2d.cuh takes
+// (3D grids). FP64 instructions bound them (2.1 M cells: 3.5 us each), so the
+// sweep is u' = gamma u + wd (f + sum_d k_d (um + up)), a missing neighbour
+// counting as zero (7 instructions with equal k_d; the operator's difference
+// form and a correction take 15), and the residual is restricted without being
+// stored: the mean over a coarse cell needs the differences across its outer
+// faces only, since what crosses an inner face cancels (7 per fine cell
+// against 15). Blocks are 32 x 8 cells of a plane.
+constexpr int kBX = 32, kBY = 8;
+
+template <int DIM>
+__device__ __forceinline__ double neighbours(const double *__restrict__ u, long long p, int i, int j, int k,
+                                             const Geo &g, const Coef &s, int &cls) {
+  const int x[3] = {i, j, k};
+  const long long st[3] = {1, g.sy, g.sz};
+  const int mul[3] = {1, 3, 9};
+  double sum[3];
+  cls = 0;
+#pragma unroll
+  for (int d = 0; d < DIM; d++) {
+    const bool lo = x[d] == 0, hi = x[d] == g.n - 1;
+    sum[d] = (lo ? 0.0 : u[p - st[d]]) + (hi ? 0.0 : u[p + st[d]]);
+    cls += mul[d] * ((int)lo + (int)hi);
+  }
+  if (s.equal) return s.k[0] * (DIM == 3 ? (sum[0] + sum[1]) + sum[2] : sum[0] + sum[1]);
+  double acc = s.k[0] * sum[0];
+#pragma unroll
+  for (int d = 1; d < DIM; d++) acc = fma(s.k[d], sum[d], acc);
+  return acc;
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(kBX * kBY) kv_rbgs_half(double *u, const double *__restrict__ f, Geo g, Coef s,
+                                                          double gamma, int color) {
+  const int j = blockIdx.y * kBY + threadIdx.y, k = DIM == 3 ? (int)blockIdx.z : 0;
+  const int i = 2 * (blockIdx.x * kBX + threadIdx.x) + ((color + j + k) & 1);
+  if (i >= g.n || j >= g.n) return;
+  const long long p = (long long)k * g.sz + (long long)j * g.sy + i;
+  int cls;
+  const double b = f[p] + neighbours<DIM>(u, p, i, j, k, g, s, cls);
+  const double v = s.wd[cls] * b;
+  u[p] = gamma != 0.0 ? fma(gamma, u[p], v) : v;
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(kBX * kBY) kv_jacobi(const double *__restrict__ uin, double *__restrict__ uout,
+                                                       const double *__restrict__ f, Geo g, Coef s, double gamma) {
+  const int i = blockIdx.x * kBX + threadIdx.x, j = blockIdx.y * kBY + threadIdx.y;
+  const int k = DIM == 3 ? (int)blockIdx.z : 0;
+  if (i >= g.n || j >= g.n) return;
+  const long long p = (long long)k * g.sz + (long long)j * g.sy + i;
+  int cls;
+  const double b = f[p] + neighbours<DIM>(uin, p, i, j, k, g, s, cls);
+  const double v = s.wd[cls] * b;
+  uout[p] = gamma != 0.0 ? fma(gamma, uin[p], v) : v;
+}
+
+// Coarse cell: f = mean of its fine cells' residuals; u = its value after the
+// first sweep (first = 1: Jacobi) or red half-sweep (2) from zero, else 0.
+template <int DIM>
+__global__ void __launch_bounds__(kBX * kBY)
+    kv_restrict(const double *__restrict__ u, const double *__restrict__ f, Geo g, Coef s, double *__restrict__ fc,
+                double *__restrict__ uc, Geo gc, Coef sc, int first) {
+  const int x[3] = {(int)(blockIdx.x * kBX + threadIdx.x), (int)(blockIdx.y * kBY + threadIdx.y),
+                    DIM == 3 ? (int)blockIdx.z : 0};
+  if (x[0] >= gc.n || x[1] >= gc.n) return;
+  const long long st[3] = {1, g.sy, g.sz};
+  const long long p = (long long)(2 * x[2]) * g.sz + (long long)(2 * x[1]) * g.sy + 2 * x[0];
+  constexpr int N = 1 << DIM;
+  double v[N], r = 0.0, su = 0.0;
+#pragma unroll
+  for (int c = 0; c < N; c++) {
+    const long long q = p + (c & 1) + ((c >> 1) & 1) * g.sy + (c >> 2) * g.sz;
+    v[c] = u[q];
+    r += f[q];
+    su += v[c];
+  }
+  r = fma(-s.sigma, su, r);
+  int cls = 0;
+  const int mul[3] = {1, 3, 9};
+#pragma unroll
+  for (int d = 0; d < DIM; d++) {
+    const bool lo = x[d] == 0, hi = x[d] == gc.n - 1;
+    double t = 0.0;
+#pragma unroll
+    for (int c = 0; c < N; c++) {
+      const long long q = p + (c & 1) + ((c >> 1) & 1) * g.sy + (c >> 2) * g.sz;
+      const bool up = (c >> d) & 1;  // the cell's outer face on this axis
+      const bool edge = up ? hi : lo;
+      const double gh = s.neumann ? v[c] : -v[c];
+      t += v[c] - (edge ? gh : u[up ? q + st[d] : q - st[d]]);
+    }
+    r = fma(-s.k[d], t, r);
+    cls += mul[d] * ((int)lo + (int)hi);
+  }
+  r *= DIM == 3 ? 0.125 : 0.25;
+  const long long P = (long long)x[2] * gc.sz + (long long)x[1] * gc.sy + x[0];
+  fc[P] = r;
+  uc[P] = first == 1 || (first == 2 && ((x[0] + x[1] + x[2]) & 1) == 0) ? sc.wd[cls] * r : 0.0;
 }
 
 // One block: assembles the coarsest operator over its N = n^DIM cells
@@ -376,6 +479,7 @@ Coef coef_of(const mg_cc_ctx *c, const Lev &L) {
   for (int d = 0; d < 3; d++) s.k[d] = c->p.c[d] * s.ih2;
   const bool neumann = c->p.bc == MG_CC_NEUMANN;
   s.neumann = neumann;
+  s.equal = c->p.c[0] == c->p.c[1] && (c->p.dim == 2 || c->p.c[0] == c->p.c[2]);
   // diag of each boundary class: per axis, a_d boundary faces (a_d = 2 only
   // for a single cell) weigh 0 (Neumann) or 2 (Dirichlet), interior faces 1
   const int dim = c->p.dim;
@@ -534,11 +638,55 @@ mg::Small2D small_desc(const mg_cc_ctx *c, int l, bool zero) {
   return d;
 }
 
+dim3 tiles(const mg_cc_ctx *c, int nx, int n) {
+  return dim3((unsigned)((nx + kBX - 1) / kBX), (unsigned)((n + kBY - 1) / kBY), c->p.dim == 3 ? (unsigned)n : 1u);
+}
+
+mg_status vcycle_rec(mg_cc_ctx *c, int l, bool zero = false, int *nparts = nullptr);
+
+// Sweeps of level l; begun: the first sweep (Jacobi) or red half-sweep is in u.
+mg_status general_smooth(mg_cc_ctx *c, int l, int sweeps, bool begun) {
+  Lev &L = c->lv[l];
+  const Geo g = geo_of(L);
+  const Coef s = coef_of(c, L);
+  const double gamma = 1.0 - c->p.omega;
+  const dim3 block(kBX, kBY);
+  if (c->p.smoother == MG_RBGS) {
+    for (int h = begun ? 1 : 0; h < 2 * sweeps; h++)
+      DIMCALL(c->p.dim, kv_rbgs_half, tiles(c, (L.n + 1) / 2, L.n), block, L.u[L.cur], L.f, g, s, gamma, h & 1);
+  } else {
+    for (int h = begun ? 1 : 0; h < sweeps; h++) {
+      DIMCALL(c->p.dim, kv_jacobi, tiles(c, L.n, L.n), block, L.u[L.cur], L.u[L.cur ^ 1], L.f, g, s, gamma);
+      L.cur ^= 1;
+    }
+  }
+  return MG_OK;
+}
+
+// One level of Algorithm 1 on the kv_ kernels. start: -1 u as it is, 0 from
+// zero, 1 u holds the first (half-)sweep from zero.
+mg_status general_cycle(mg_cc_ctx *c, int l, int start) {
+  mg_status st;
+  Lev &L = c->lv[l], &C = c->lv[l + 1];
+  if (start == 0) CCK(cudaMemsetAsync(L.u[L.cur], 0, (size_t)L.count * sizeof(double), c->s));
+  if ((st = general_smooth(c, l, c->p.nu1, start == 1 && c->p.nu1 > 0))) return st;
+  // the next level: u from its first sweep unless it solves, or starts by itself
+  const bool last = l + 2 == c->nl, own = !last && (small_desc(c, l + 1, true).lg > 0 || level_fx(c, l + 1));
+  const int first = last || own || c->p.nu1 == 0 ? 0 : c->p.smoother == MG_RBGS ? 2 : 1;
+  DIMCALL(c->p.dim, kv_restrict, tiles(c, C.n, C.n), dim3(kBX, kBY), L.u[L.cur], L.f, geo_of(L), coef_of(c, L), C.f,
+          C.u[C.cur], geo_of(C), coef_of(c, C), first);
+  if (last) st = op_coarse(c);
+  else if (own) st = vcycle_rec(c, l + 1, true);
+  else st = general_cycle(c, l + 1, 1);
+  if (st || (st = op_prolong(c, l))) return st;
+  return general_smooth(c, l, c->p.nu2, false);
+}
+
 // Algorithm 1 from level l down; coarse levels start from zero (`zero`: u_l
 // counts as zero whatever its buffer holds). nparts (finest level, may be
 // NULL): the number of partial sums of the squared residual that the last
 // pass left in c->partials, 0 if it left none.
-mg_status vcycle_rec(mg_cc_ctx *c, int l, bool zero = false, int *nparts = nullptr) {
+mg_status vcycle_rec(mg_cc_ctx *c, int l, bool zero, int *nparts) {
   mg_status st;
   Lev &L = c->lv[l];
   if (nparts) *nparts = 0;
@@ -569,14 +717,11 @@ mg_status vcycle_rec(mg_cc_ctx *c, int l, bool zero = false, int *nparts = nullp
       if ((st = fx_pass(c, l, left > 2 ? 2 : left, false, false, false, nullptr))) return st;
     return MG_OK;
   }
-  if (zero) CCK(cudaMemsetAsync(L.u[L.cur], 0, (size_t)L.count * sizeof(double), c->s));
-  if (l == c->nl - 1) return op_coarse(c);
-  if ((st = op_smooth(c, l, c->p.nu1))) return st;
-  if ((st = op_residual(c, l))) return st;
-  if ((st = op_restrict(c, l))) return st;
-  if ((st = vcycle_rec(c, l + 1, true))) return st;
-  if ((st = op_prolong(c, l))) return st;
-  return op_smooth(c, l, c->p.nu2);
+  if (l == c->nl - 1) {
+    if (zero) CCK(cudaMemsetAsync(L.u[L.cur], 0, (size_t)L.count * sizeof(double), c->s));
+    return op_coarse(c);
+  }
+  return general_cycle(c, l, zero ? 0 : -1);
 }
 
 mg_status level_ok(const mg_cc_ctx *c, int level, bool need_coarser) {
