@@ -20,6 +20,7 @@
 
 #include "mg_cd.h"
 #include "mg_internal.h"
+#include "stepgraph.h"
 
 namespace mg {
 namespace cd {
@@ -385,6 +386,7 @@ struct mg_cd_ctx {
   // run on the kr_ kernels. A call that sets or reads faces, sets f or works on
   // one level first expands the faces (to_complex).
   bool phased;
+  mg::StepGraphs graphs;
 };
 
 namespace {
@@ -594,6 +596,27 @@ mg_status vcycle_rec(mg_cd_ctx *c, int l) {
   return op_smooth(c, l, c->p.nu2);
 }
 
+// Step k of a solve: a V-cycle and the residual norm.
+mg_status solve_step(mg_cd_ctx *c, int k) {
+  int status = 0;
+  CDK(mg::step(
+      c->graphs, k, c->s,
+      [&] {
+        unsigned b = c->phased ? 1u << 31 : 0u;
+        for (int l = 0; l < c->nl; l++) b |= (unsigned)c->lv[l].cur << l;
+        return b;
+      },
+      [&](unsigned b) {
+        for (int l = 0; l < c->nl; l++) c->lv[l].cur = (b >> l) & 1u;
+      },
+      [&]() -> int {
+        mg_status st = vcycle_rec(c, 0);
+        return st ? st : op_norm(c, 0);
+      },
+      &status));
+  return (mg_status)status;
+}
+
 mg_status level_ok(const mg_cd_ctx *c, int level, bool need_coarser) {
   if (!c) return cdfail(MG_EINVAL, "NULL context");
   if (level < 0 || level >= c->nl - (need_coarser ? 1 : 0)) return cdfail(MG_EINVAL, "level %d out of range", level);
@@ -677,6 +700,7 @@ mg_status mg_cd_create(const mg_cd_params *p, void *arena, size_t arena_bytes, m
 }
 
 mg_status mg_cd_destroy(mg_cd_ctx *c) {
+  if (c) mg::drop(c->graphs);
   free(c);
   return MG_OK;
 }
@@ -788,7 +812,7 @@ mg_status mg_cd_solve(mg_cd_ctx *c, double tol, int *iters, double *relres, doub
   int k = 0;
   double rho = r0 > 0.0 ? 1.0 : 0.0;
   while (r0 > 0.0 && rho > tol && k < c->p.maxit) {
-    if ((st = vcycle_rec(c, 0)) || (st = op_norm(c, 0))) return st;
+    if ((st = solve_step(c, k))) return st;
     double rk;
     if ((st = read_norm(c, &rk))) return st;
     rho = rk / r0;

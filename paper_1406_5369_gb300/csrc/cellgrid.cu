@@ -23,6 +23,7 @@
 #include "fx2d.cuh"
 #include "mg_cc.h"
 #include "mg_internal.h"
+#include "stepgraph.h"
 
 namespace mg {
 namespace cc {
@@ -388,6 +389,7 @@ struct mg_cc_ctx {
   double *partials;  // mg::kMaxPartials norm partial sums
   double *norm_out;  // one double
   cudaStream_t s;
+  mg::StepGraphs graphs;
 };
 
 namespace {
@@ -724,6 +726,28 @@ mg_status vcycle_rec(mg_cc_ctx *c, int l, bool zero, int *nparts) {
   return general_cycle(c, l, zero ? 0 : -1);
 }
 
+// Step k of a solve: a V-cycle and the residual norm.
+mg_status solve_step(mg_cc_ctx *c, int k) {
+  int status = 0;
+  CCK(mg::step(
+      c->graphs, k, c->s,
+      [&] {
+        unsigned b = 0;
+        for (int l = 0; l < c->nl; l++) b |= (unsigned)c->lv[l].cur << l;
+        return b;
+      },
+      [&](unsigned b) {
+        for (int l = 0; l < c->nl; l++) c->lv[l].cur = (b >> l) & 1u;
+      },
+      [&]() -> int {
+        int np = 0;
+        mg_status st = vcycle_rec(c, 0, false, &np);
+        return st ? st : np ? norm_final(c, np) : op_norm(c, 0);
+      },
+      &status));
+  return (mg_status)status;
+}
+
 mg_status level_ok(const mg_cc_ctx *c, int level, bool need_coarser) {
   if (!c) return ccfail(MG_EINVAL, "NULL context");
   if (level < 0 || level >= c->nl - (need_coarser ? 1 : 0))
@@ -794,6 +818,7 @@ mg_status mg_cc_create(const mg_cc_params *p, void *arena, size_t arena_bytes, m
 }
 
 mg_status mg_cc_destroy(mg_cc_ctx *c) {
+  if (c) mg::drop(c->graphs);
   free(c);
   return MG_OK;
 }
@@ -883,8 +908,7 @@ mg_status mg_cc_solve(mg_cc_ctx *c, double tol, int *iters, double *relres, doub
   int k = 0;
   double rho = r0 > 0.0 ? 1.0 : 0.0;
   while (r0 > 0.0 && rho > tol && k < c->p.maxit) {
-    int np = 0;
-    if ((st = vcycle_rec(c, 0, false, &np)) || (st = np ? norm_final(c, np) : op_norm(c, 0))) return st;
+    if ((st = solve_step(c, k))) return st;
     double rk;
     if ((st = read_norm(c, &rk))) return st;
     rho = rk / r0;
