@@ -136,6 +136,9 @@ cudaError_t norm_stream(const Level &L, const void *u, const void *f, double *pa
 // meaning of their 2D namespaces' counterparts; partial sums are per block.
 namespace d3 {
 bool z_ok(const Level &L);
+// Single-problem operators of a level take them: FP64 levels up to 65^3 are too
+// small to march through (33^3: 16 us an operator, one thread per node 2 us).
+bool z_march(const Level &L);
 bool transfer_ok(const Level &F, const Level &C);
 cudaError_t z_sweep(const Level &L, const void *uin, void *uout, const void *f, int color, double omega,
                     cudaStream_t s);

@@ -134,6 +134,8 @@ cudaError_t launch_stencil(z3::Args3 a, long long max_blocks, int *nblocks, cuda
 
 bool z_ok(const Level &L) { return L.dim == 3 && !L.kf[0] && L.n >= 5; }
 
+bool z_march(const Level &L) { return z_ok(L) && !(L.dtype == F64 && L.n <= 65); }
+
 cudaError_t z_sweep(const Level &L, const void *uin, void *uout, const void *f, int color, double omega,
                     cudaStream_t s) {
   z3::Args3 a = stencil_args(L, omega);
