@@ -33,8 +33,8 @@
 // 52 are written and the rows before a chunk are 1.3 times the minimal work),
 // then HBM (400 MB at 6.7 TB/s: 60 us). 4097^2, V(2,2), one cycle's level in
 // us, FP64 kernels -> these: red-black omega = 1, fused FP64 passes and norm
-// 1062 -> 200 (pre), 654 + 378 -> 246 (post with the norm); Jacobi, one kernel
-// per operator, 1453 -> 247, 1294 + 398 -> 298.
+// 1062 -> 191 (pre), 654 + 378 -> 234 (post with the norm); Jacobi, one kernel
+// per operator, 1453 -> 235, 1294 + 398 -> 283.
 //
 // The same pass serves node-based grids (values on boundary nodes stay, full
 // weighting, bilinear interpolation) and cell-centred ones (a missing
@@ -102,14 +102,15 @@ __device__ __forceinline__ long long mul62(long long x, Mul m) {
 }
 
 // X m / 2^62 for a residual: returns the product's integer part and takes
-// its next kLoBits bits off lo (no bias: a one-sided error of one unit in
+// its next BITS bits off lo (no bias: a one-sided error of one unit in
 // every residual would grow by n^2 / 16 in the solution).
+template <int BITS>
 __device__ __forceinline__ long long mul62(long long x, Mul m, int &lo) {
   const int xh = (int)(x >> 32);
   const unsigned xl = (unsigned)x;
   const long long mid = (long long)((unsigned long long)xl * (unsigned)m.hi) + (long long)xh * m.lo +
                         (((long long)xl * m.lo) >> 32);
-  lo -= (int)(((unsigned)mid & 0x3fffffffu) >> (30 - kLoBits));
+  lo -= (int)(((unsigned)mid & 0x3fffffffu) >> (30 - BITS));
   return (((long long)xh * m.hi) << 2) + (mid >> 30);
 }
 
@@ -133,14 +134,15 @@ __device__ __forceinline__ long long to_fix(double x, int E, int P) {
   const long long sg = (long long)(__double2hiint(x) >> 31);
   return (v ^ sg) - sg;
 }
-// The same with kLoBits further bits in lo (same sign as x).
+// The same with BITS further bits in lo (same sign as x).
+template <int BITS>
 __device__ __forceinline__ long long to_fix2(double x, int E, int P, int &lo) {
   const unsigned long long y = significand(x, P - 53);
-  const int t = E - expo(x), t2 = t - kLoBits;
+  const int t = E - expo(x), t2 = t - BITS;
   const unsigned q = t2 >= 0 ? (unsigned)shr64(y, (unsigned)t2) : (unsigned)y << -t2;
   const int sg = __double2hiint(x) >> 31;
   const long long v = (long long)shr64(y, (unsigned)t);
-  lo = ((int)(q & ((1u << kLoBits) - 1)) ^ sg) - sg;
+  lo = ((int)(q & ((1u << BITS) - 1)) ^ sg) - sg;
   return (v ^ (long long)sg) - (long long)sg;
 }
 // x 2^(E - 1022 - P), rounded to nearest. The conversion instruction issues
@@ -225,7 +227,7 @@ __device__ __forceinline__ bool strip(const Args &a, unsigned char *ring, int la
   const bool ccol_ok = c0 >= 0 && J0 < a.nc;
   const bool out_lane = lane >= kHalo / kVec && lane < 32 - kHalo / kVec && col_ok;
   const int r0 = ch * a.R, r1 = min(r0 + a.R, n);
-  const int tstart = max(r0 - 8, 0);
+  const int tstart = max(r0 - kHalo, 0);
   const int tend = OUT == kNone ? r1 - 1 + S : r1 + S;
   unsigned char *su = ring + lane * LB;
   unsigned char *sf = su + (ZERO ? 0 : kRing * 32 * LB);
@@ -359,7 +361,7 @@ __device__ __forceinline__ bool strip(const Args &a, unsigned char *ring, int la
       for (int q = 0; q < kVec; q++) {
         if constexpr (FX) {
           U[0][q] = ZERO ? 0 : to_fix(ud[q], E, P);
-          F[0][q] = to_fix2(fd[q], E - a.fexp, P, FL[0][q]);
+          F[0][q] = to_fix2<kLoBits>(fd[q], E - a.fexp, P, FL[0][q]);
         } else {
           U[0][q] = ud[q];
           F[0][q] = fd[q] * a.fpow;
@@ -468,11 +470,11 @@ __device__ __forceinline__ bool strip(const Args &a, unsigned char *ring, int la
             rr[q] = F[sc][q] + (uw + ue) + (us + un) - (kx + ky) * u;
           } else {
             long long tx = kx * u - (uw + ue), ty = ky * u - (us + un);
-            if (a.has_px) tx = mul62(tx, a.px, lo2);
-            if (a.has_py) ty = mul62(ty, a.py, lo2);
+            if (a.has_px) tx = mul62<kLoBits>(tx, a.px, lo2);
+            if (a.has_py) ty = mul62<kLoBits>(ty, a.py, lo2);
             rr[q] = F[sc][q] - (tx + ty);
           }
-          if (CELL && a.has_s) rr[q] -= mul62(u, a.s, lo2);
+          if (CELL && a.has_s) rr[q] -= mul62<kLoBits>(u, a.s, lo2);
           if (ok) rl[q] = lo2;
         } else {
           const N tx = (u - uw) + (u - ue) + (kx - 2) * u, ty = (u - us) + (u - un) + (ky - 2) * u;
@@ -589,7 +591,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_fx2d(const __grid_cons
   if (gw >= (long long)a.nstrips * a.nchunks) return;
   const int s = (int)(gw % a.nstrips), ch = (int)(gw / a.nstrips);
   const int x0 = s * kOut - kHalo, r0 = ch * a.R, r1 = min(r0 + a.R, a.n);
-  const int tstart = max(r0 - 8, 0), tend = r1 + S;
+  const int tstart = max(r0 - kHalo, 0), tend = r1 + S;
   const int tlast = tstart + ((tend - tstart) / kGroup + 1) * kGroup - 1;
   const bool interior = x0 >= 1 && x0 + kCols - 1 <= a.n - 2 && tstart - S - 2 >= 1 && tlast <= a.n - 2;
   unsigned char *ring = smem + (size_t)wib * WB;
@@ -676,11 +678,12 @@ inline bool set_operator(Args &a, double kx, double ky, double sigma, int edge, 
   return a.P >= 54;
 }
 
-// Rows per chunk: one wave of resident warps, a multiple of 8.
+// Rows per chunk: one wave of resident warps, an even number (multiples of 8
+// left 6 % of the resident warps without a chunk at 4097^2).
 inline int chunk_rows(int n, int nstrips, long long warps) {
   long long chunks = warps / nstrips;
   if (chunks < 1) chunks = 1;
-  const int R = ((int)((n + chunks - 1) / chunks) + 7) / 8 * 8;
+  const int R = ((int)((n + chunks - 1) / chunks) + 1) / 2 * 2;
   return R < 8 ? 8 : R;
 }
 

@@ -1,4 +1,4 @@
-"""The fixed-point 2D passes of the FP64 levels against the oracle's FP64
+"""The fixed-point 2D passes and the other FP64 cycles against the oracle's FP64
 V-cycles and the per-operator kernels (fuse=False).
 
 Tolerances: per-cycle relative residuals to 1e-12 (the bound of the FP64
@@ -188,5 +188,31 @@ def test_cell_cluster_cycle_matches_oracle(n, bc, sigma, smoother, omega, nu, nc
     ref.set_rhs(f)
     ref.set_u(u0)
     rho = ref.solve(0.0, 3)
+    assert np.max(np.abs(hist - rho) / np.maximum(1.0, rho)) <= 1e-12, (hist, rho)
+    assert rel_err(s.get_field(0, "u"), ref.get_u()) <= 1e-12
+
+
+# 3D cells: sums over the outer faces of coarse cells, first half-sweep from zero
+@pytest.mark.parametrize("n,bc,sigma,smoother,omega,nu,c", [
+    (64, "neumann", 3000.0, "rbgs", 1.0, (2, 2), (1.0, 1.0, 1.0)),
+    (64, "dirichlet", 0.0, "rbgs", 1.1, (2, 1), (1.0, 1.0, 1.0)),
+    (128, "neumann", 1.0, "jacobi", 0.8, (3, 2), (1.0, 1.0, 1.0)),
+    (128, "dirichlet", 100.0, "rbgs", 1.0, (1, 3), (0.8, 1.25, 1.0)),
+    (64, "neumann", 10.0, "jacobi", 0.8, (2, 2), (1.25, 0.9, 0.9)),
+    (8, "neumann", 1.0, "rbgs", 1.0, (0, 2), (1.0, 1.0, 1.0)),
+    (4, "dirichlet", 0.0, "jacobi", 0.8, (1, 0), (1.0, 1.0, 1.0)),
+])
+def test_cell_3d_cycles_match_oracle(n, bc, sigma, smoother, omega, nu, c):
+    need_gpu()
+    from paper_1406_5369_gb300 import CCSolver
+    f, u0 = synth.uniform(21, (n, n, n)) - 0.5, synth.uniform(22, (n, n, n))
+    s = CCSolver(3, n, c=c, sigma=sigma, bc=bc, smoother=smoother, omega=omega, nu1=nu[0], nu2=nu[1], maxit=2)
+    s.set_rhs(f)
+    s.set_solution(u0)
+    _, _, hist = s.solve(0.0, raise_on_noconv=False)
+    ref = oracle.CCHierarchy(3, n, c=c, sigma=sigma, bc=bc, smoother=SM[smoother], omega=omega, nu1=nu[0], nu2=nu[1])
+    ref.set_rhs(f)
+    ref.set_u(u0)
+    rho = ref.solve(0.0, 2)
     assert np.max(np.abs(hist - rho) / np.maximum(1.0, rho)) <= 1e-12, (hist, rho)
     assert rel_err(s.get_field(0, "u"), ref.get_u()) <= 1e-12
