@@ -358,6 +358,23 @@ bool level_fx(const mg_ctx *c, int l) {
          c->lv[l + 1].dtype == mg::F64 && mg::d2::fx_ok(L, (int)c->opt.smoother, c->opt.omega);
 }
 
+// True when level l runs on the fixed-point 3D passes (fx3d.cuh).
+bool level_fx3(const mg_ctx *c, int l) {
+  return c->opt.fuse && !c->dc && c->dim == 3 && l + 1 < c->nl && c->opt.nu1 >= 1 && c->opt.nu2 >= 1 &&
+         c->lv[l + 1].dtype == mg::F64 && mg::d3::fx_ok(c->lv[l], (int)c->opt.smoother, c->opt.omega);
+}
+
+// One fixed-point pass (one sweep) of level l from the live solution buffer to the other.
+mg_status fx3_pass(mg_ctx *c, int l, int kind, bool zero, bool corr, bool restr, int *nparts, cudaStream_t s) {
+  Level &L = c->lv[l], &C = c->lv[l + 1];
+  TLAUNCH(c, kind, l, s,
+          mg::d3::fx_pass(L, &C, (int)c->opt.smoother, c->opt.omega, L.u[L.cur], L.u[L.cur ^ 1], zero,
+                          corr ? C.u[C.cur] : nullptr, restr ? C.f : nullptr, nparts ? c->partials : nullptr, nparts,
+                          s));
+  L.cur ^= 1;
+  return MG_OK;
+}
+
 // The cluster V-cycle of levels l .. nl-1 (small2d.cuh); lg = 0 when the
 // context or the level does not take it. cluster_max_n sets its largest level.
 mg::Small2D small_desc(const mg_ctx *c, int l, bool zero) {
@@ -446,6 +463,15 @@ mg_status vcycle_rec(mg_ctx *c, int l, bool zero, cudaStream_t s, int *nparts = 
     if ((st = fx_pass(c, l, MG_KERNEL_POSTSMOOTH, first, false, true, false, left ? nullptr : nparts, s))) return st;
     for (; left > 0; left -= 2)
       if ((st = fx_pass(c, l, MG_KERNEL_POSTSMOOTH, left > 2 ? 2 : left, false, false, false, nullptr, s))) return st;
+    return MG_OK;
+  }
+  if (level_fx3(c, l)) {
+    for (int k = 0; k < c->opt.nu1; k++)
+      if ((st = fx3_pass(c, l, MG_KERNEL_PRESMOOTH, zero && k == 0, false, k + 1 == c->opt.nu1, nullptr, s))) return st;
+    if ((st = vcycle_rec(c, l + 1, true, s))) return st;
+    for (int k = 0; k < c->opt.nu2; k++)
+      if ((st = fx3_pass(c, l, MG_KERNEL_POSTSMOOTH, false, k == 0, false, k + 1 == c->opt.nu2 ? nparts : nullptr, s)))
+        return st;
     return MG_OK;
   }
   if (level_fused(c, l)) {

@@ -115,6 +115,16 @@ cudaError_t fx_pass(const Level &L, const Level *C, int smoother, double omega, 
                     bool zero, const void *ec, void *fc, double *partials, int *nparts, int rows, cudaStream_t s);
 }  // namespace d2
 
+// The same for 3D levels (fx3d.cuh), one sweep per pass; below 257^3 the
+// tiles' recomputed edges cost more than the FP64 arithmetic they save (a level
+// of 129^3, V(2,2): 299 us against 284 us).
+namespace d3 {
+constexpr int kFxMinN = 257, kFxMaxN = 1025;
+bool fx_ok(const Level &L, int smoother, double omega);
+cudaError_t fx_pass(const Level &L, const Level *C, int smoother, double omega, const void *uin, void *uout, bool zero,
+                    const void *ec, void *fc, double *partials, int *nparts, cudaStream_t s);
+}  // namespace d3
+
 // Streaming 2D finest-level kernels (constant stencil). dc_step: FP64 outer
 // step of defect correction (optional update u_out = u_in + e, residual ->
 // defect d, per-warp partial sums); norm_stream: per-warp partial sums of
