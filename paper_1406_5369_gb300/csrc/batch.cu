@@ -26,6 +26,7 @@
 
 #include "ctx.h"
 #include "kernels.cuh"
+#include "dcvar2d.cuh"
 #include "outer2d.cuh"
 #include "stencil3d.cuh"
 
@@ -228,6 +229,15 @@ __global__ void kb_dc_residual(const BOuter *__restrict__ os) {
     if (o.d) st((Ti *)o.d + q, oz::d2f_bits(r));  // truncation to FP32 without the FP64 pipe
   });
   acc = block_sum(acc);
+  if (threadIdx.x == 0) o.partials[blockIdx.x] = acc;
+}
+
+// The same for 2D problems with a variable stencil, on the integer pipes.
+template <typename Ti> __global__ void __launch_bounds__(dv2::kThreads) kb_dc_residual_var2d(const BOuter *__restrict__ os) {
+  const BOuter &o = os[blockIdx.y];
+  if (gone(o)) return;
+  const dv2::Prob a = {o.u, o.f, o.sd.kf0, o.sd.kf1, o.d, o.sd.inv_h2, o.go.n, o.go.sy, o.gi.sy};
+  const double acc = dv2::residual<Ti, false>(a);
   if (threadIdx.x == 0) o.partials[blockIdx.x] = acc;
 }
 
@@ -1041,8 +1051,8 @@ mg_status batched_outer(mg_batch *b, const std::vector<mg_ctx *> &ps, bool updat
     // read u and f (FP64) and the FP64 faces, write the defect
     BTimer tm(b, MG_BATCH_OUTER, gnodes * (16.0 + wi + (var ? 8.0 * dim : 0.0)));
     if (dim == 2) {
-      if (ti == F32) { if (var) kb_dc_residual<2, float, true><<<gr, 256, 0, s>>>(dev); else kb_dc_residual<2, float, false><<<gr, 256, 0, s>>>(dev); }
-      else { if (var) kb_dc_residual<2, bf16, true><<<gr, 256, 0, s>>>(dev); else kb_dc_residual<2, bf16, false><<<gr, 256, 0, s>>>(dev); }
+      if (ti == F32) { if (var) kb_dc_residual_var2d<float><<<gr, dv2::kThreads, 0, s>>>(dev); else kb_dc_residual<2, float, false><<<gr, 256, 0, s>>>(dev); }
+      else { if (var) kb_dc_residual_var2d<bf16><<<gr, dv2::kThreads, 0, s>>>(dev); else kb_dc_residual<2, bf16, false><<<gr, 256, 0, s>>>(dev); }
     } else {
       if (ti == F32) { if (var) kb_dc_residual<3, float, true><<<gr, 256, 0, s>>>(dev); else kb_dc_residual<3, float, false><<<gr, 256, 0, s>>>(dev); }
       else { if (var) kb_dc_residual<3, bf16, true><<<gr, 256, 0, s>>>(dev); else kb_dc_residual<3, bf16, false><<<gr, 256, 0, s>>>(dev); }

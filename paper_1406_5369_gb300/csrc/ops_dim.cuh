@@ -1,11 +1,12 @@
 // Host-side dispatch from a Level (runtime dim/dtype/stencil kind) to the
 // templated kernels. Included once per dimension with MG_DIM and MG_NS set.
+#include "dcvar2d.cuh"
 #include "kernels.cuh"
 
 namespace mg {
 namespace MG_NS {
 
-static const int kDim = MG_DIM;
+static constexpr int kDim = MG_DIM;
 
 static dim3 node_grid(int n, int bx) {
   return dim3((unsigned)((n + bx - 1) / bx), (unsigned)n, kDim == 3 ? (unsigned)n : 1u);
@@ -130,21 +131,28 @@ cudaError_t coarse_dense(const Level &L, void *u, const void *f, cudaStream_t s)
   return cudaGetLastError();
 }
 
+// 2D, variable stencil, on the integer pipes (dcvar2d.cuh).
+template <typename Ti>
+__global__ void __launch_bounds__(dv2::kThreads) k_dc_residual_var2d(const dv2::Prob a, double *__restrict__ partials) {
+  const double acc = dv2::residual<Ti, true>(a);
+  if (threadIdx.x == 0) partials[blockIdx.x] = acc;
+}
+
 cudaError_t dc_residual(const Level &O, const void *u, const void *f, const Level &I, void *d, double *partials,
                         int nblocks, cudaStream_t s) {
-  bool var = O.kf[0] != nullptr;
-  Sten<double> st = sten_of<double>(O);
-  switch (I.dtype) {
-    case F32:
-      if (var) k_dc_residual<kDim, float, true><<<nblocks, 256, 0, s>>>((const double *)u, (const double *)f, geo_of(O), st, (float *)d, geo_of(I), partials);
-      else k_dc_residual<kDim, float, false><<<nblocks, 256, 0, s>>>((const double *)u, (const double *)f, geo_of(O), st, (float *)d, geo_of(I), partials);
-      break;
-    case BF16:
-      if (var) k_dc_residual<kDim, bf16, true><<<nblocks, 256, 0, s>>>((const double *)u, (const double *)f, geo_of(O), st, (bf16 *)d, geo_of(I), partials);
-      else k_dc_residual<kDim, bf16, false><<<nblocks, 256, 0, s>>>((const double *)u, (const double *)f, geo_of(O), st, (bf16 *)d, geo_of(I), partials);
-      break;
-    default:
-      return cudaErrorInvalidValue;
+  if (I.dtype != F32 && I.dtype != BF16) return cudaErrorInvalidValue;
+  const Sten<double> st = sten_of<double>(O);
+  const double *uo = (const double *)u, *fo = (const double *)f;
+  if (!O.kf[0]) {
+    if (I.dtype == F32) k_dc_residual<kDim, float, false><<<nblocks, 256, 0, s>>>(uo, fo, geo_of(O), st, (float *)d, geo_of(I), partials);
+    else k_dc_residual<kDim, bf16, false><<<nblocks, 256, 0, s>>>(uo, fo, geo_of(O), st, (bf16 *)d, geo_of(I), partials);
+  } else if constexpr (kDim == 2) {
+    const dv2::Prob a = {uo, fo, st.kf0, st.kf1, d, O.inv_h2, O.n, O.pitch, I.pitch};
+    if (I.dtype == F32) k_dc_residual_var2d<float><<<nblocks, dv2::kThreads, 0, s>>>(a, partials);
+    else k_dc_residual_var2d<bf16><<<nblocks, dv2::kThreads, 0, s>>>(a, partials);
+  } else {
+    if (I.dtype == F32) k_dc_residual<kDim, float, true><<<nblocks, 256, 0, s>>>(uo, fo, geo_of(O), st, (float *)d, geo_of(I), partials);
+    else k_dc_residual<kDim, bf16, true><<<nblocks, 256, 0, s>>>(uo, fo, geo_of(O), st, (bf16 *)d, geo_of(I), partials);
   }
   return cudaGetLastError();
 }
