@@ -387,7 +387,7 @@ struct mg_cc_ctx {
   Lev lv[kMaxLev];
   double *ainv;      // coarsest grid inverse, N x N
   double *partials;  // mg::kMaxPartials norm partial sums
-  double *norm_out;  // one double
+  double *norm_out;  // the norm (and its square)
   cudaStream_t s;
   mg::StepGraphs graphs;
 };
@@ -467,7 +467,7 @@ size_t layout(mg_cc_ctx *c, char *base) {
   const size_t N = (size_t)nc * nc * (dim == 3 ? nc : 1);
   c->ainv = take(N * N * sizeof(double));
   c->partials = take(mg::kMaxPartials * sizeof(double));
-  c->norm_out = take(sizeof(double));
+  c->norm_out = take(2 * sizeof(double));
   return align256(off);
 }
 
@@ -644,6 +644,8 @@ dim3 tiles(const mg_cc_ctx *c, int nx, int n) {
   return dim3((unsigned)((nx + kBX - 1) / kBX), (unsigned)((n + kBY - 1) / kBY), c->p.dim == 3 ? (unsigned)n : 1u);
 }
 
+// A cycle that leaves the residual norm itself in c->norm_out sets *nparts to this.
+constexpr int kNormDone = -1;
 mg_status vcycle_rec(mg_cc_ctx *c, int l, bool zero = false, int *nparts = nullptr);
 
 // Sweeps of level l; begun: the first sweep (Jacobi) or red half-sweep is in u.
@@ -695,8 +697,11 @@ mg_status vcycle_rec(mg_cc_ctx *c, int l, bool zero, int *nparts) {
   {
     mg::Small2D d = small_desc(c, l, zero);
     if (d.lg > 0 && mg::small2d_ok(d)) {
-      if (nparts) d.partials = c->partials;
-      CCK(mg::small2d_cycle(d, nparts, c->s));
+      if (nparts) {
+        d.norm_out = c->norm_out;
+        *nparts = kNormDone;
+      }
+      CCK(mg::small2d_cycle(d, c->s));
       return MG_OK;
     }
   }
@@ -742,7 +747,7 @@ mg_status solve_step(mg_cc_ctx *c, int k) {
       [&]() -> int {
         int np = 0;
         mg_status st = vcycle_rec(c, 0, false, &np);
-        return st ? st : np ? norm_final(c, np) : op_norm(c, 0);
+        return st || np == kNormDone ? st : np ? norm_final(c, np) : op_norm(c, 0);
       },
       &status));
   return (mg_status)status;

@@ -417,7 +417,8 @@ mg_status fx_pass(mg_ctx *c, int l, int kind, int nu, bool zero, bool corr, bool
 // of a defect-correction step), which lets the fused kernels skip reading it.
 // `nparts` (finest level, may be NULL): a level whose last pass also forms
 // the residual leaves the partial sums of its square in c->partials and their
-// number here, otherwise 0.
+// number here (or the norm itself in c->norm_out, kNormDone), otherwise 0.
+constexpr int kNormDone = -1;
 mg_status vcycle_rec(mg_ctx *c, int l, bool zero, cudaStream_t s, int *nparts = nullptr) {
   NvtxRange range(c->level_name[l]);
   mg_status st;
@@ -425,8 +426,11 @@ mg_status vcycle_rec(mg_ctx *c, int l, bool zero, cudaStream_t s, int *nparts = 
   {
     mg::Small2D d = small_desc(c, l, zero);
     if (d.lg > 0 && mg::small2d_ok(d)) {
-      if (nparts) d.partials = c->partials;
-      TLAUNCH(c, MG_KERNEL_COARSE, l, s, mg::small2d_cycle(d, nparts, s));
+      if (nparts) {
+        d.norm_out = c->norm_out;
+        *nparts = kNormDone;
+      }
+      TLAUNCH(c, MG_KERNEL_COARSE, l, s, mg::small2d_cycle(d, s));
       return MG_OK;
     }
   }
@@ -634,6 +638,7 @@ mg_status record(mg_ctx *c, int kind, cudaStream_t s) {
   if (!c->dc) {
     int np = 0;
     if ((st = vcycle_rec(c, 0, false, s, kind == 1 ? &np : nullptr))) return st;
+    if (kind == 1 && np == kNormDone) return MG_OK;
     if (kind == 1 && np > 0) {
       TLAUNCH(c, MG_KERNEL_NORM, 0, s,
               mg::norm_finalize_ex(c->partials, np, c->norm_out, nullptr, nullptr, interior_count(c->lv[0]), s));

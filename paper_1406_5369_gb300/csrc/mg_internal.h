@@ -235,12 +235,12 @@ struct Small2D {
   double *u;
   int pitch;
   const double *dense;   // coarsest inverse, NULL for a single node
-  double *partials;      // sums of the squared residual of the result, one per block (NULL: none)
+  double *norm_out;      // norm of the result's residual and its square, two doubles (NULL: none)
 };
 constexpr int kSmallTopLog = 7;  // largest level taken by default
 void small2d_probe();
 bool small2d_ok(const Small2D &d);
-cudaError_t small2d_cycle(const Small2D &d, int *nparts, cudaStream_t s);
+cudaError_t small2d_cycle(const Small2D &d, cudaStream_t s);
 
 // Sets the message mg_last_error() returns on the calling thread.
 void set_error_message(const char *msg);

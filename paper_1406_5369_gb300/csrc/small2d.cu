@@ -69,7 +69,7 @@ size_t fill(const Small2D &d, int nctas, sm2::Args &a) {
   a.pitch_top = d.pitch;
   a.kinv = 1.0 / k;
   a.k2 = k * k;
-  a.partials = d.partials;
+  a.norm_out = d.norm_out;
   auto rows = [&](int l) { return (1 << (d.lg - l)) - (d.cell ? 0 : 1); };
   if (nd > 0) {
     const int m = rows(nd);
@@ -141,11 +141,10 @@ bool small2d_ok(const Small2D &d) {
   return g_nctas > 0 && fill(d, g_nctas, a) != 0;
 }
 
-cudaError_t small2d_cycle(const Small2D &d, int *nparts, cudaStream_t s) {
+cudaError_t small2d_cycle(const Small2D &d, cudaStream_t s) {
   sm2::Args a;
   const size_t smem = g_nctas > 0 ? fill(d, g_nctas, a) : 0;
   if (!smem) return cudaErrorInvalidValue;
-  if (nparts) *nparts = a.nctas;
   return d.cell ? launch<true>(a, smem, s) : launch<false>(a, smem, s);
 }
 

@@ -27,10 +27,11 @@
 // whose boundary faces then only change the diagonal (weights kx, ky = edge
 // instead of 2 on u).
 //
-// Measured per V(2,1) cycle from 129^2: 61 us, one launch, in place of 184 us in
-// five (block tiles for 129^2 and 65^2, the single-block cycle below). About
-// 20 us are barriers (0.5 us each), the rest FP64 issue: a level of 257^2 taken
-// along would add 40 us where the streaming passes take 36.
+// Measured per V(2,1) cycle from 129^2, with the residual norm: 54 us, one
+// launch, in place of 232 us in seven (block tiles for 129^2 and 65^2, the
+// single-block cycle below, the norm). About 20 us are barriers (0.5 us each),
+// the rest FP64 issue: 33^2 on all blocks instead of block 0 saved 5 us, a level
+// of 257^2 taken along would add 40 us where the streaming passes take 35.
 //
 // Every block executes the same sequence of cluster barriers (the loop bounds
 // are kernel arguments), and no block touches another's shared memory after
@@ -49,7 +50,7 @@ namespace cg = cooperative_groups;
 constexpr int kThreads = 512;
 constexpr int kMaxCTAs = 16;
 constexpr int kTopLog = 8;    // largest level: 2^8 cells (257 nodes) per dimension
-constexpr int kLocalLog = 5;  // levels up to 2^5 cells run in block 0
+constexpr int kLocalLog = 4;  // levels up to 2^4 cells run in block 0
 constexpr int kMaxDist = kTopLog - kLocalLog, kMaxLocal = kLocalLog + 1;
 
 struct Lev {
@@ -73,7 +74,7 @@ struct Args {
   const double *dense;  // inverse of the coarsest operator, NULL for one node
   double dense_k;       // coarsest k: the inverse acts on f = f' k
   double one;           // one node: u = f' one
-  double *partials;     // block r's sum of the squared top residual (NULL: none)
+  double *norm_out;     // norm of the top residual and its square (NULL: none)
   double k2;            // top k squared
   int total;            // elements of shared memory
 };
@@ -314,18 +315,19 @@ template <bool CELL> __global__ void __launch_bounds__(kThreads, 1) k_small2d(co
     smooth<CELL, false>(a, cl, sm, l, r, x, a.nu2);
   }
   if (a.nd == 0 && top_swapped && a.nl > 1) { double *t = x.U; x.U = x.V; x.V = t; }
+  __shared__ double sums[kMaxCTAs];  // block 0: every block's sum of squares
   if (a.nd > 0 || r == 0) {
     double acc = 0.0;
     for (int q = threadIdx.x; q < (x.R << x.lg); q += kThreads) {
       const int jl = q >> x.lg, i = (q & ((1 << x.lg) - 1)) + 1;
       if (i > x.m) continue;
       a.u_top[(long long)(x.b0 + jl - off) * a.pitch_top + i - off] = x.U[(jl + 1) * x.pitch + i];
-      if (a.partials) {
+      if (a.norm_out) {
         const double v = resid<CELL>(a, a.lv[0], x, jl, i);
         acc += v * v;
       }
     }
-    if (a.partials) {
+    if (a.norm_out) {
       __shared__ double part[kThreads / 32];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -334,11 +336,17 @@ template <bool CELL> __global__ void __launch_bounds__(kThreads, 1) k_small2d(co
       if (threadIdx.x == 0) {
         double t = 0.0;
         for (int w = 0; w < kThreads / 32; w++) t += part[w];
-        a.partials[r] = t * a.k2;
+        *cl.map_shared_rank(&sums[r], 0) = t;
       }
     }
   }
   cl.sync();
+  if (a.norm_out && r == 0 && threadIdx.x == 0) {
+    double t = 0.0;
+    for (int b = 0; b < a.nctas; b++) t += sums[b];
+    a.norm_out[0] = sqrt(t * a.k2);
+    a.norm_out[1] = t * a.k2;
+  }
 }
 
 }  // namespace sm2
