@@ -130,6 +130,9 @@ typedef struct { int kind; const double *dirichlet_values; } mg_boundary;
  *                         33 and below in one of them); 0 = 257, values
  *                         below 129 = never (per-level kernels and the
  *                         single-block cycle below 65)
+ *                         FP64, 2D constant stencil, either smoother: the
+ *                         largest level from which one cluster runs the rest of
+ *                         the V-cycle in FP64; 0 = 129, at most 257 counts
  * canary                : 1 = debug layout: every buffer the context lays out
  *                         in the arena is followed by a 256-byte guard zone
  *                         filled with the byte 0xA5 at mg_create and checked
