@@ -253,15 +253,10 @@ __global__ void __launch_bounds__(kBX * kBY) kv_jacobi(const double *__restrict_
   uout[p] = gamma != 0.0 ? fma(gamma, uin[p], v) : v;
 }
 
-// Coarse cell: f = mean of its fine cells' residuals; u = its value after the
-// first sweep (first = 1: Jacobi) or red half-sweep (2) from zero, else 0.
+// Mean of the residuals of the fine cells of coarse cell x (nc per dimension).
 template <int DIM>
-__global__ void __launch_bounds__(kBX * kBY)
-    kv_restrict(const double *__restrict__ u, const double *__restrict__ f, Geo g, Coef s, double *__restrict__ fc,
-                double *__restrict__ uc, Geo gc, Coef sc, int first) {
-  const int x[3] = {(int)(blockIdx.x * kBX + threadIdx.x), (int)(blockIdx.y * kBY + threadIdx.y),
-                    DIM == 3 ? (int)blockIdx.z : 0};
-  if (x[0] >= gc.n || x[1] >= gc.n) return;
+__device__ __forceinline__ double restricted(const double *__restrict__ u, const double *__restrict__ f, const Geo &g,
+                                             const Coef &s, const int (&x)[3], int nc) {
   const long long st[3] = {1, g.sy, g.sz};
   const long long p = (long long)(2 * x[2]) * g.sz + (long long)(2 * x[1]) * g.sy + 2 * x[0];
   constexpr int N = 1 << DIM;
@@ -274,11 +269,9 @@ __global__ void __launch_bounds__(kBX * kBY)
     su += v[c];
   }
   r = fma(-s.sigma, su, r);
-  int cls = 0;
-  const int mul[3] = {1, 3, 9};
 #pragma unroll
   for (int d = 0; d < DIM; d++) {
-    const bool lo = x[d] == 0, hi = x[d] == gc.n - 1;
+    const bool lo = x[d] == 0, hi = x[d] == nc - 1;
     double t = 0.0;
 #pragma unroll
     for (int c = 0; c < N; c++) {
@@ -289,12 +282,117 @@ __global__ void __launch_bounds__(kBX * kBY)
       t += v[c] - (edge ? gh : u[up ? q + st[d] : q - st[d]]);
     }
     r = fma(-s.k[d], t, r);
-    cls += mul[d] * ((int)lo + (int)hi);
   }
-  r *= DIM == 3 ? 0.125 : 0.25;
+  return r * (DIM == 3 ? 0.125 : 0.25);
+}
+
+// u of a cell after the first sweep (first = 1: Jacobi) or red half-sweep (2)
+// from zero, else 0.
+template <int DIM>
+__device__ __forceinline__ double first_sweep(double f, const Coef &s, const int (&x)[3], int n, int first) {
+  const int mul[3] = {1, 3, 9};
+  int cls = 0;
+#pragma unroll
+  for (int d = 0; d < DIM; d++) cls += mul[d] * ((int)(x[d] == 0) + (int)(x[d] == n - 1));
+  return first == 1 || (first == 2 && ((x[0] + x[1] + x[2]) & 1) == 0) ? s.wd[cls] * f : 0.0;
+}
+
+// Coarse cell: f = mean of its fine cells' residuals; u = first_sweep.
+template <int DIM>
+__global__ void __launch_bounds__(kBX * kBY)
+    kv_restrict(const double *__restrict__ u, const double *__restrict__ f, Geo g, Coef s, double *__restrict__ fc,
+                double *__restrict__ uc, Geo gc, Coef sc, int first) {
+  const int x[3] = {(int)(blockIdx.x * kBX + threadIdx.x), (int)(blockIdx.y * kBY + threadIdx.y),
+                    DIM == 3 ? (int)blockIdx.z : 0};
+  if (x[0] >= gc.n || x[1] >= gc.n) return;
+  const double r = restricted<DIM>(u, f, g, s, x, gc.n);
   const long long P = (long long)x[2] * gc.sz + (long long)x[1] * gc.sy + x[0];
   fc[P] = r;
-  uc[P] = first == 1 || (first == 2 && ((x[0] + x[1] + x[2]) & 1) == 0) ? sc.wd[cls] * r : 0.0;
+  uc[P] = first_sweep<DIM>(r, sc, x, gc.n, first);
+}
+
+// V-cycle of the 3D levels of at most 8^3 cells in one block, one thread per
+// cell of the largest: some 10 launches of 2 us per level otherwise.
+constexpr int kSmall3 = 8, kSmall3Lev = 4, kSmall3Threads = kSmall3 * kSmall3 * kSmall3;
+struct Small3 {
+  int nl, nu1, nu2, jacobi, start;  // start: as general_cycle's
+  double gamma;
+  Coef s[kSmall3Lev];
+  int n[kSmall3Lev];
+  const double *f, *ainv;
+  double *u;
+  Geo g;  // of the top level's global fields
+};
+__global__ void __launch_bounds__(kSmall3Threads) kv_small3(const __grid_constant__ Small3 a) {
+  __shared__ double U[2][kSmall3Lev][kSmall3Threads], F[kSmall3Lev][kSmall3Threads];
+  const int t = threadIdx.x;
+  int cur[kSmall3Lev];
+  auto cell = [&](int l, int (&x)[3]) {
+    const int n = a.n[l];
+    x[0] = t % n;
+    x[1] = (t / n) % n;
+    x[2] = t / (n * n);
+    return t < n * n * n;
+  };
+  auto smooth = [&](int l, int sweeps, bool begun) {
+    const Geo g = {a.n[l], a.n[l], (long long)a.n[l] * a.n[l]};
+    int x[3];
+    const bool mine = cell(l, x);
+    for (int h = begun ? 1 : 0; h < (a.jacobi ? sweeps : 2 * sweeps); h++) {
+      const double *u = U[cur[l]][l];
+      double *out = U[a.jacobi ? cur[l] ^ 1 : cur[l]][l];
+      if (mine && (a.jacobi || ((x[0] + x[1] + x[2]) & 1) == (h & 1))) {
+        int cls;
+        const double b = F[l][t] + neighbours<3>(u, t, x[0], x[1], x[2], g, a.s[l], cls);
+        out[t] = fma(a.gamma, u[t], a.s[l].wd[cls] * b);
+      }
+      if (a.jacobi) cur[l] ^= 1;
+      __syncthreads();
+    }
+  };
+  const int first = a.nu1 == 0 ? 0 : a.jacobi ? 1 : 2;
+#pragma unroll
+  for (int l = 0; l < kSmall3Lev; l++) cur[l] = 0;
+  int x[3];
+  long long top = 0;
+  if (cell(0, x)) {
+    top = (long long)x[2] * a.g.sz + (long long)x[1] * a.g.sy + x[0];
+    F[0][t] = a.f[top];
+    U[0][0][t] = a.start == 0 ? first_sweep<3>(F[0][t], a.s[0], x, a.n[0], first) : a.u[top];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int l = 0; l < kSmall3Lev - 1; l++) {
+    if (l + 1 >= a.nl) break;
+    smooth(l, a.nu1, a.nu1 > 0 && (l > 0 || a.start >= 0));
+    if (cell(l + 1, x)) {
+      const Geo g = {a.n[l], a.n[l], (long long)a.n[l] * a.n[l]};
+      const double r = restricted<3>(U[cur[l]][l], F[l], g, a.s[l], x, a.n[l + 1]);
+      F[l + 1][t] = r;
+      U[0][l + 1][t] = l + 2 == a.nl ? 0.0 : first_sweep<3>(r, a.s[l + 1], x, a.n[l + 1], first);
+    }
+    __syncthreads();
+  }
+  {
+    const int l = a.nl - 1, N = a.n[l] * a.n[l] * a.n[l];
+    if (t < N) {
+      double acc = 0.0;
+      for (int q = 0; q < N; q++) acc += a.ainv[q * N + t] * F[l][q];
+      U[0][l][t] = acc;
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int l = kSmall3Lev - 2; l >= 0; l--) {
+    if (l + 1 >= a.nl) continue;
+    if (cell(l, x)) {
+      const int m = a.n[l + 1];
+      U[cur[l]][l][t] += U[cur[l + 1]][l + 1][((x[2] >> 1) * m + (x[1] >> 1)) * m + (x[0] >> 1)];
+    }
+    __syncthreads();
+    smooth(l, a.nu2, false);
+  }
+  if (cell(0, x)) a.u[top] = U[cur[0]][0][t];
 }
 
 // One block: assembles the coarsest operator over its N = n^DIM cells
@@ -672,6 +770,27 @@ mg_status general_smooth(mg_cc_ctx *c, int l, int sweeps, bool begun) {
 mg_status general_cycle(mg_cc_ctx *c, int l, int start) {
   mg_status st;
   Lev &L = c->lv[l], &C = c->lv[l + 1];
+  if (c->p.dim == 3 && L.n <= kSmall3 && c->nl - l <= kSmall3Lev) {
+    Small3 a;
+    memset(&a, 0, sizeof a);
+    a.nl = c->nl - l;
+    for (int i = 0; i < a.nl; i++) {
+      a.s[i] = coef_of(c, c->lv[l + i]);
+      a.n[i] = c->lv[l + i].n;
+    }
+    a.nu1 = c->p.nu1;
+    a.nu2 = c->p.nu2;
+    a.jacobi = c->p.smoother != MG_RBGS;
+    a.start = start;
+    a.gamma = 1.0 - c->p.omega;
+    a.f = L.f;
+    a.u = L.u[L.cur];
+    a.g = geo_of(L);
+    a.ainv = c->ainv;
+    kv_small3<<<1, kSmall3Threads, 0, c->s>>>(a);
+    CCK(cudaGetLastError());
+    return MG_OK;
+  }
   if (start == 0) CCK(cudaMemsetAsync(L.u[L.cur], 0, (size_t)L.count * sizeof(double), c->s));
   if ((st = general_smooth(c, l, c->p.nu1, start == 1 && c->p.nu1 > 0))) return st;
   // the next level: u from its first sweep unless it solves, or starts by itself

@@ -200,6 +200,9 @@ def test_cell_cluster_cycle_matches_oracle(n, bc, sigma, smoother, omega, nu, nc
     (128, "dirichlet", 100.0, "rbgs", 1.0, (1, 3), (0.8, 1.25, 1.0)),
     (64, "neumann", 10.0, "jacobi", 0.8, (2, 2), (1.25, 0.9, 0.9)),
     (8, "neumann", 1.0, "rbgs", 1.0, (0, 2), (1.0, 1.0, 1.0)),
+    (8, "dirichlet", 3.0, "jacobi", 0.8, (2, 0), (1.0, 2.0, 1.0)),
+    (16, "neumann", 2.0, "jacobi", 0.8, (3, 2), (1.0, 1.0, 1.0)),
+    (32, "dirichlet", 0.0, "rbgs", 1.3, (1, 2), (1.0, 1.0, 0.6)),
     (4, "dirichlet", 0.0, "jacobi", 0.8, (1, 0), (1.0, 1.0, 1.0)),
 ])
 def test_cell_3d_cycles_match_oracle(n, bc, sigma, smoother, omega, nu, c):
