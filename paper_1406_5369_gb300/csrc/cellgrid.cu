@@ -50,7 +50,6 @@ struct Coef {
   double k[3];        // c_d / h^2 = c_d n^2 (exact scaling: n is a power of two)
   double sigma, ih2;  // ih2 = 1/h^2 = n^2
   int neumann;        // ghost value u_p (Neumann) or -u_p (Dirichlet)
-  int equal;          // the k[d] are the same
   double wd[27];      // omega / diag by boundary class a_0 + 3 a_1 + 9 a_2
 };
 
@@ -199,32 +198,30 @@ template <int DIM> __device__ __forceinline__ void coarse_cell(int t, int n, int
 // Kernels of the V-cycle on levels that neither fx2d.cuh nor small2d.cuh takes
 // (3D grids). FP64 instructions bound them (2.1 M cells: 3.5 us each), so the
 // sweep is u' = gamma u + wd (f + sum_d k_d (um + up)), a missing neighbour
-// counting as zero (7 instructions with equal k_d; the operator's difference
+// counting as zero (7 instructions; the operator's difference
 // form and a correction take 15), and the residual is restricted without being
 // stored: the mean over a coarse cell needs the differences across its outer
 // faces only, since what crosses an inner face cancels (7 per fine cell
 // against 15). Blocks are 32 x 8 cells of a plane.
 constexpr int kBX = 32, kBY = 8;
 
+// f_p + sum_d k_d (um + up), one FMA per neighbour (an FP64 addition issues
+// slower than an FMA here: 76 cycles of a scheduler against 64).
 template <int DIM>
-__device__ __forceinline__ double neighbours(const double *__restrict__ u, long long p, int i, int j, int k,
+__device__ __forceinline__ double neighbours(const double *__restrict__ u, double f, long long p, int i, int j, int k,
                                              const Geo &g, const Coef &s, int &cls) {
   const int x[3] = {i, j, k};
   const long long st[3] = {1, g.sy, g.sz};
   const int mul[3] = {1, 3, 9};
-  double sum[3];
   cls = 0;
 #pragma unroll
   for (int d = 0; d < DIM; d++) {
     const bool lo = x[d] == 0, hi = x[d] == g.n - 1;
-    sum[d] = (lo ? 0.0 : u[p - st[d]]) + (hi ? 0.0 : u[p + st[d]]);
+    f = fma(s.k[d], lo ? 0.0 : u[p - st[d]], f);
+    f = fma(s.k[d], hi ? 0.0 : u[p + st[d]], f);
     cls += mul[d] * ((int)lo + (int)hi);
   }
-  if (s.equal) return s.k[0] * (DIM == 3 ? (sum[0] + sum[1]) + sum[2] : sum[0] + sum[1]);
-  double acc = s.k[0] * sum[0];
-#pragma unroll
-  for (int d = 1; d < DIM; d++) acc = fma(s.k[d], sum[d], acc);
-  return acc;
+  return f;
 }
 
 template <int DIM>
@@ -235,7 +232,7 @@ __global__ void __launch_bounds__(kBX * kBY) kv_rbgs_half(double *u, const doubl
   if (i >= g.n || j >= g.n) return;
   const long long p = (long long)k * g.sz + (long long)j * g.sy + i;
   int cls;
-  const double b = f[p] + neighbours<DIM>(u, p, i, j, k, g, s, cls);
+  const double b = neighbours<DIM>(u, f[p], p, i, j, k, g, s, cls);
   const double v = s.wd[cls] * b;
   u[p] = gamma != 0.0 ? fma(gamma, u[p], v) : v;
 }
@@ -248,7 +245,7 @@ __global__ void __launch_bounds__(kBX * kBY) kv_jacobi(const double *__restrict_
   if (i >= g.n || j >= g.n) return;
   const long long p = (long long)k * g.sz + (long long)j * g.sy + i;
   int cls;
-  const double b = f[p] + neighbours<DIM>(uin, p, i, j, k, g, s, cls);
+  const double b = neighbours<DIM>(uin, f[p], p, i, j, k, g, s, cls);
   const double v = s.wd[cls] * b;
   uout[p] = gamma != 0.0 ? fma(gamma, uin[p], v) : v;
 }
@@ -343,7 +340,7 @@ __global__ void __launch_bounds__(kSmall3Threads) kv_small3(const __grid_constan
       double *out = U[a.jacobi ? cur[l] ^ 1 : cur[l]][l];
       if (mine && (a.jacobi || ((x[0] + x[1] + x[2]) & 1) == (h & 1))) {
         int cls;
-        const double b = F[l][t] + neighbours<3>(u, t, x[0], x[1], x[2], g, a.s[l], cls);
+        const double b = neighbours<3>(u, F[l][t], t, x[0], x[1], x[2], g, a.s[l], cls);
         out[t] = fma(a.gamma, u[t], a.s[l].wd[cls] * b);
       }
       if (a.jacobi) cur[l] ^= 1;
@@ -579,7 +576,6 @@ Coef coef_of(const mg_cc_ctx *c, const Lev &L) {
   for (int d = 0; d < 3; d++) s.k[d] = c->p.c[d] * s.ih2;
   const bool neumann = c->p.bc == MG_CC_NEUMANN;
   s.neumann = neumann;
-  s.equal = c->p.c[0] == c->p.c[1] && (c->p.dim == 2 || c->p.c[0] == c->p.c[2]);
   // diag of each boundary class: per axis, a_d boundary faces (a_d = 2 only
   // for a single cell) weigh 0 (Neumann) or 2 (Dirichlet), interior faces 1
   const int dim = c->p.dim;
