@@ -1,9 +1,9 @@
 // Implicit Euler steps of nonlinear complex diffusion (include/mg_cd.h):
 // Sec. 4's second test problem on cell-centred grids, complex FP64.
 //
-// Layout: level l has n_l = n / 2^l cells per dimension and eight complex
+// Layout: level l has n_l = n / 2^l cells per dimension and seven complex
 // fields (double2: real, imaginary) u[0], u[1] (Jacobi ping-pong), f, r, the
-// face coefficients gx, gy, wd = omega / diag and gf = wd f per cell, rows padded to 128
+// face coefficients gx, gy and wd = omega / diag per cell, rows padded to 128
 // bytes (pitch = n_l rounded up to 8 complex values), x fastest, no ghost
 // cells. One thread per cell (per cell of the swept colour for red-black
 // Gauss-Seidel), rows on blockIdx.y. The arithmetic is FP64 throughout and
@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(kThreads) kr_norm_partials(const double2 *__re
 }
 
 // Faces: general complex coefficients in gx, gy, or (phased, see the context)
-// real weights in gx and the smoother's q in gy.
+// real weights in gx, the smoother's q in gy and its g = wd f in r.
 struct Lev {
   int n, pitch;
   long long count;
@@ -383,8 +383,8 @@ struct mg_cd_ctx {
   double *partials, *norm_out;
   cudaStream_t s;
   // The faces are e^{i theta} times real weights (set by begin_step): V-cycles
-  // run on the kr_ kernels. A call that sets or reads faces, sets f or works on
-  // one level first expands the faces (to_complex).
+  // run on the kr_ kernels. A call that sets or reads faces, sets f or r, reads r
+  // or works on one level first expands the faces (to_complex).
   bool phased;
   mg::StepGraphs graphs;
 };
@@ -448,7 +448,7 @@ size_t layout(mg_cd_ctx *c, char *base) {
     L.gx = (double2 *)take(bytes);
     L.gy = (double2 *)take(bytes);
     L.wd = (double2 *)take(bytes);
-    L.gf = (double2 *)take(bytes);
+    L.gf = L.r;
     if (n == 1) break;
   }
   c->partials = (double *)take(kNormBlocks * sizeof(double));
@@ -718,7 +718,7 @@ mg_status mg_cd_set_field(mg_cd_ctx *c, int level, int field, const double *src)
   if (!src) return cdfail(MG_EINVAL, "src is NULL");
   double2 *dst = field_ptr(c->lv[level], field);
   if (!dst) return cdfail(MG_EINVAL, "unknown field %d", field);
-  if (field != MG_CD_U && field != MG_CD_R && (st = to_complex(c))) return st;
+  if (field != MG_CD_U && (st = to_complex(c))) return st;
   if ((st = copy_in(c, c->lv[level], dst, src))) return st;
   return (field == MG_CD_GX || field == MG_CD_GY) ? op_wdiag(c, level) : MG_OK;
 }
@@ -730,6 +730,7 @@ mg_status mg_cd_get_field(mg_cd_ctx *c, int level, int field, double *dst) {
   Lev &L = c->lv[level];
   const double2 *src = field_ptr(L, field);
   if (!src) return cdfail(MG_EINVAL, "unknown field %d", field);
+  if (field == MG_CD_R && c->phased && ((st = to_complex(c)) || (st = op_residual(c, level)))) return st;
   if ((field == MG_CD_GX || field == MG_CD_GY) && (st = to_complex(c))) return st;
   CDK(cudaMemcpy2DAsync(dst, (size_t)L.n * 16, src, (size_t)L.pitch * 16, (size_t)L.n * 16, (size_t)L.n,
                         cudaMemcpyDefault, c->s));

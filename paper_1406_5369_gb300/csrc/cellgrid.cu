@@ -481,7 +481,7 @@ struct mg_cc_ctx {
   int nl;
   Lev lv[kMaxLev];
   double *ainv;      // coarsest grid inverse, N x N
-  double *partials;  // mg::kMaxPartials norm partial sums
+  double *partials;  // kNormBlocks norm partial sums
   double *norm_out;  // the norm (and its square)
   cudaStream_t s;
   mg::StepGraphs graphs;
@@ -561,8 +561,8 @@ size_t layout(mg_cc_ctx *c, char *base) {
   const int nc = c->lv[c->nl - 1].n;
   const size_t N = (size_t)nc * nc * (dim == 3 ? nc : 1);
   c->ainv = take(N * N * sizeof(double));
-  c->partials = take(mg::kMaxPartials * sizeof(double));
-  c->norm_out = take(2 * sizeof(double));
+  c->partials = take(kNormBlocks * sizeof(double));
+  c->norm_out = take(sizeof(double));  // the rounding up to 256 bytes below leaves room for its square beside it
   return align256(off);
 }
 
@@ -698,6 +698,7 @@ mg_status fx_pass(mg_cc_ctx *c, int l, int nu, bool zero, bool corr, bool restr,
   a.ec = corr ? C.u[C.cur] : nullptr;
   a.fc = restr ? C.f : nullptr;
   a.partials = nparts ? c->partials : nullptr;
+  a.max_parts = kNormBlocks;
   a.n = L.n;
   a.pitch = L.pitch;
   a.nc = C.n;

@@ -32,6 +32,7 @@ cudaError_t fx_pass(const Level &L, const Level *C, int smoother, double omega, 
   a.ec = (const double *)ec;
   a.fc = (double *)fc;
   a.partials = partials;
+  a.max_parts = kMaxPartials;
   a.n = L.n;
   a.pitch = L.pitch;
   if (C) {

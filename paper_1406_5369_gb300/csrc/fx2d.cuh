@@ -77,6 +77,7 @@ struct Args {
   double *uout, *fc, *partials;  // kNorm: one partial sum per warp
   int n, pitch, nc, pitchc;
   int R, nstrips, nchunks;
+  int max_parts;       // room for the partial sums of kNorm
   int P;               // bits of the largest loaded value
   int fexp, fbound;    // f' = (f fscale) 2^fexp, one of the two trivial; the exponent of f' is at most f's + fbound
   double fscale, fpow; // fpow = 2^fexp
@@ -705,7 +706,7 @@ cudaError_t launch(Args a, int rows, int *nparts, cudaStream_t s) {
   a.nstrips = (a.n + kOut - 1) / kOut;
   a.R = rows > 0 ? (rows + 7) / 8 * 8 : chunk_rows(a.n, a.nstrips, wave);
   if (OUT == kNorm)  // one partial sum per warp
-    while ((long long)a.nstrips * ((a.n + a.R - 1) / a.R) > kMaxPartials) a.R += 8;
+    while ((long long)a.nstrips * ((a.n + a.R - 1) / a.R) > a.max_parts) a.R += 8;
   a.nchunks = (a.n + a.R - 1) / a.R;
   const long long warps = (long long)a.nstrips * a.nchunks;
   if (nparts) *nparts = (int)warps;
