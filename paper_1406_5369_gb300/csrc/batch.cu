@@ -236,7 +236,8 @@ __global__ void kb_dc_residual(const BOuter *__restrict__ os) {
 template <typename Ti> __global__ void __launch_bounds__(dv2::kThreads) kb_dc_residual_var2d(const BOuter *__restrict__ os) {
   const BOuter &o = os[blockIdx.y];
   if (gone(o)) return;
-  const dv2::Prob a = {o.u, o.f, o.sd.kf0, o.sd.kf1, o.d, o.sd.inv_h2, o.go.n, o.go.sy, o.gi.sy};
+  const dv2::Prob a = {o.u, o.f, o.sd.kf0, o.sd.kf1, o.d, o.sd.inv_h2, o.go.n, o.go.sy, o.gi.sy,
+                       dv2::batch_rows(o.go.n)};
   const double acc = dv2::residual<Ti, false>(a);
   if (threadIdx.x == 0) o.partials[blockIdx.x] = acc;
 }
@@ -1030,6 +1031,11 @@ mg_status batched_outer(mg_batch *b, const std::vector<mg_ctx *> &ps, bool updat
     b->launches++;
   }
   if (!gen.empty()) {
+    // 2D variable stencils: the small problems first, they keep the FP64 kernel
+    size_t small = gen.size();
+    if (dim == 2 && var)
+      small = std::stable_partition(gen.begin(), gen.end(), [](const BOuter &g) { return g.go.n < dv2::kBatchMinN; }) -
+              gen.begin();
     const BOuter *dev = (const BOuter *)push(b, gen.data(), sizeof(BOuter) * gen.size());
     if (!dev) return bfail(MG_ENOMEM, "batch descriptor area exhausted");
     dim3 gr(kPartBlocks, (unsigned)gen.size());
@@ -1051,8 +1057,20 @@ mg_status batched_outer(mg_batch *b, const std::vector<mg_ctx *> &ps, bool updat
     // read u and f (FP64) and the FP64 faces, write the defect
     BTimer tm(b, MG_BATCH_OUTER, gnodes * (16.0 + wi + (var ? 8.0 * dim : 0.0)));
     if (dim == 2) {
-      if (ti == F32) { if (var) kb_dc_residual_var2d<float><<<gr, dv2::kThreads, 0, s>>>(dev); else kb_dc_residual<2, float, false><<<gr, 256, 0, s>>>(dev); }
-      else { if (var) kb_dc_residual_var2d<bf16><<<gr, dv2::kThreads, 0, s>>>(dev); else kb_dc_residual<2, bf16, false><<<gr, 256, 0, s>>>(dev); }
+      const dim3 gs(kPartBlocks, (unsigned)small);
+      if (!var) {
+        if (ti == F32) kb_dc_residual<2, float, false><<<gr, 256, 0, s>>>(dev);
+        else kb_dc_residual<2, bf16, false><<<gr, 256, 0, s>>>(dev);
+      } else if (small > 0) {
+        if (ti == F32) kb_dc_residual<2, float, true><<<gs, 256, 0, s>>>(dev);
+        else kb_dc_residual<2, bf16, true><<<gs, 256, 0, s>>>(dev);
+      }
+      if (var && small < gen.size()) {
+        const dim3 gl(kPartBlocks, (unsigned)(gen.size() - small));
+        if (ti == F32) kb_dc_residual_var2d<float><<<gl, dv2::kThreads, 0, s>>>(dev + small);
+        else kb_dc_residual_var2d<bf16><<<gl, dv2::kThreads, 0, s>>>(dev + small);
+        if (small > 0) b->launches++;
+      }
     } else {
       if (ti == F32) { if (var) kb_dc_residual<3, float, true><<<gr, 256, 0, s>>>(dev); else kb_dc_residual<3, float, false><<<gr, 256, 0, s>>>(dev); }
       else { if (var) kb_dc_residual<3, bf16, true><<<gr, 256, 0, s>>>(dev); else kb_dc_residual<3, bf16, false><<<gr, 256, 0, s>>>(dev); }

@@ -34,7 +34,17 @@ namespace dv2 {
 
 constexpr int kWarps = 4, kThreads = 32 * kWarps;
 constexpr int kOut = 60;   // columns written per strip
-constexpr int kRows = 40;  // rows per chunk: the largest problem of a batch has a chunk for each of its 512 warps
+// Rows per chunk of a batch's problems. A warp walks its chunk alone (0.7 us a
+// row), so problems with few strips take short ones; the largest (1025^2) has a
+// chunk for each of its 512 warps. Below kBatchMinN a problem's rows are too few
+// to hide a chunk's latency (100 problems of 65^2: 3.41 ms a solve on the FP64
+// kernel, 3.49 ms here; 20 of 129^2 to 513^2: 8.51 and 8.41 ms).
+constexpr int kBatchMinN = 257;
+__host__ __device__ constexpr int batch_rows(int n) { return n <= 257 ? 8 : n <= 513 ? 16 : 40; }
+// A problem alone: short chunks, or too few warps; below 1025^2 the FP64 kernel's
+// one node per thread is as fast (129^2: 738 us a solve, 750 us with this one).
+constexpr int kAloneMinN = 1025;
+constexpr int alone_rows(int n) { return n <= 1025 ? 8 : n <= 2049 ? 16 : 40; }
 constexpr int kP = 56;
 
 struct Prob {
@@ -43,9 +53,10 @@ struct Prob {
   double ih2;
   int n;
   long long sy, syi;  // row strides of the FP64 fields and of the defect
+  int rows;           // per chunk
 };
 
-inline __host__ __device__ int tasks(int n) { return ((n + kOut - 1) / kOut) * ((n - 2 + kRows - 1) / kRows); }
+__device__ __forceinline__ int tasks(const Prob &a) { return ((a.n + kOut - 1) / kOut) * ((a.n - 2 + a.rows - 1) / a.rows); }
 
 // Flux of a difference through a face with coefficient k >= 0: x k / 2^(e -
 // 1023) * 4, e its biased exponent (of the product of the low words only the
@@ -77,7 +88,7 @@ template <typename Ti, bool RN> __device__ __forceinline__ void put(Ti *p, doubl
 template <typename Ti, bool RN> __device__ __forceinline__ double task(const Prob &a, int t, int lane) {
   const int n = a.n, strips = (n + kOut - 1) / kOut;
   const int c0 = (t % strips) * kOut - 2 + 2 * lane;
-  const int r0 = 1 + (t / strips) * kRows, r1 = min(r0 + kRows, n - 1);  // rows r0 .. r1 - 1
+  const int R = a.rows, r0 = 1 + (t / strips) * R, r1 = min(r0 + R, n - 1);  // rows r0 .. r1 - 1
   const bool out = lane >= 1 && lane < 31;
   const bool ok0 = out && c0 >= 1 && c0 <= n - 2, ok1 = out && c0 + 1 >= 1 && c0 + 1 <= n - 2;
   const bool ld_ok = c0 >= 0 && c0 < n;  // rows are padded to an even number of columns
@@ -196,7 +207,7 @@ template <typename Ti, bool RN> __device__ __forceinline__ double task(const Pro
 
 // One problem by the blocks of a grid row; the block's sum of squares, valid in thread 0.
 template <typename Ti, bool RN> __device__ __forceinline__ double residual(const Prob &a) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, count = tasks(a.n);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, count = tasks(a);
   double acc = 0.0;
   for (int t = blockIdx.x * kWarps + w; t < count; t += gridDim.x * kWarps) acc += task<Ti, RN>(a, t, lane);
   return block_sum(acc);

@@ -146,8 +146,8 @@ cudaError_t dc_residual(const Level &O, const void *u, const void *f, const Leve
   if (!O.kf[0]) {
     if (I.dtype == F32) k_dc_residual<kDim, float, false><<<nblocks, 256, 0, s>>>(uo, fo, geo_of(O), st, (float *)d, geo_of(I), partials);
     else k_dc_residual<kDim, bf16, false><<<nblocks, 256, 0, s>>>(uo, fo, geo_of(O), st, (bf16 *)d, geo_of(I), partials);
-  } else if constexpr (kDim == 2) {
-    const dv2::Prob a = {uo, fo, st.kf0, st.kf1, d, O.inv_h2, O.n, O.pitch, I.pitch};
+  } else if (kDim == 2 && O.n >= dv2::kAloneMinN) {
+    const dv2::Prob a = {uo, fo, st.kf0, st.kf1, d, O.inv_h2, O.n, O.pitch, I.pitch, dv2::alone_rows(O.n)};
     if (I.dtype == F32) k_dc_residual_var2d<float><<<nblocks, dv2::kThreads, 0, s>>>(a, partials);
     else k_dc_residual_var2d<bf16><<<nblocks, dv2::kThreads, 0, s>>>(a, partials);
   } else {

@@ -32,7 +32,7 @@ def coefficients(kind, n):
     return np.where(g > 0.5, 1e8, 1.0)  # eight orders of magnitude between neighbours
 
 
-# 5: less than a strip; 33, 129: ragged strips and chunks; 1025: many chunks per block row
+# alone, 1025 is the smallest size on the integer kernel; the others keep the FP64 one
 @pytest.mark.parametrize("n", [5, 9, 33, 129, 1025])
 @pytest.mark.parametrize("kind", ["lognormal", "jump"])
 @pytest.mark.parametrize("precision", ["fp32_dc", "bf16_dc"])
@@ -53,7 +53,7 @@ def test_outer_residual(n, kind, precision):
 @pytest.mark.parametrize("shift", [-900, 700])
 def test_magnitudes_outside_the_range(shift):
     """u beyond the exponent range of the scale: the same residual, scaled."""
-    n = 65
+    n = 1025
     k = coefficients("lognormal", n)
     f, u = synth.uniform_rhs(2, n, 55), synth.uniform(56, (n, n))
     u[0], u[-1], u[:, 0], u[:, -1] = 0, 0, 0, 0
@@ -66,7 +66,7 @@ def test_magnitudes_outside_the_range(shift):
 
 @pytest.mark.parametrize("where", ["u", "f"])
 def test_non_finite_values_stay_where_they_are(where):
-    n = 129
+    n = 1025
     k = coefficients("lognormal", n)
     f, u = synth.uniform_rhs(2, n, 57), synth.uniform(58, (n, n))
     u[0], u[-1], u[:, 0], u[:, -1] = 0, 0, 0, 0
@@ -77,3 +77,22 @@ def test_non_finite_values_stay_where_they_are(where):
     assert np.array_equal(np.isfinite(d)[1:-1, 1:-1], np.isfinite(r)[1:-1, 1:-1])
     ok = np.isfinite(r)
     assert np.abs(d[ok] - r[ok]).max() <= 1e-6 * np.abs(r[ok]).max()
+
+
+def test_batch_of_every_size():
+    """Sizes on both kernels of the batch engine (257 is the smallest on the integer one)."""
+    need_gpu()
+    from paper_1406_5369_gb300 import BatchSolver, Solver
+    sizes = [5, 9, 33, 65, 129, 257, 513, 1025]
+    ks = [np.where(coefficients("jump", n) > 1, 30.0, 1.0) for n in sizes]
+    fs = [synth.uniform_rhs(2, n, 70 + n) for n in sizes]
+    solvers = [Solver(2, n, k=k, precision="fp32_dc", inner_cycles=2, maxit=40) for n, k in zip(sizes, ks)]
+    b = BatchSolver(len(sizes))
+    for s, f in zip(solvers, fs):
+        s.set_rhs(f)
+        s.set_solution(None)
+        b.add(s)
+    b.solve(1e-9, maxit=40)
+    for s, f, k in zip(solvers, fs, ks):
+        r = oracle.residual(s.get_solution(), f, faces=oracle.node_faces(k))
+        assert oracle.norm(r) <= 1.01e-9 * oracle.norm(f)
