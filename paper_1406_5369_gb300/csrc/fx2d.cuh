@@ -154,6 +154,13 @@ __device__ __forceinline__ double to_dbl(long long x, int E, int P) {
   return __hiloint2double(x == 0 ? 0 : hi, __double2loint(d));
 }
 
+// x as to_dbl stores it: rounded to 53 bits. A pass that forms the norm rounds
+// each node's last update with it, so that the norm is that of the stored
+// solution: the bits beyond FP64 would hide its rounding (4097^2, smooth data,
+// at the rounding floor: 0.09 of the residual of what was returned). Both
+// conversions issue on the FP64 pipe.
+__device__ __forceinline__ long long stored(long long x) { return __double2ll_rn(__ll2double_rn(x)); }
+
 __device__ __forceinline__ long long shup(long long v) { return __shfl_up_sync(0xffffffffu, v, 1); }
 __device__ __forceinline__ long long shdn(long long v) { return __shfl_down_sync(0xffffffffu, v, 1); }
 __device__ __forceinline__ int shup(int v) { return __shfl_up_sync(0xffffffffu, v, 1); }
@@ -411,6 +418,8 @@ __device__ __forceinline__ bool strip(const Args &a, unsigned char *ring, int la
                                        Old[JAC ? h : 0][q] + U[h - 1][q], cls_of(r, c0 + q));
 #pragma unroll
         for (int q = 0; q < kVec; q++) {
+          if constexpr (FX && OUT == kNorm)
+            if (h == S) nv[q] = stored(nv[q]);
           Old[JAC ? h : 0][q] = U[h][q];  // the row's values before this sweep, for the row below
           if (rin && in(c0 + q)) U[h][q] = nv[q];
         }
@@ -418,7 +427,9 @@ __device__ __forceinline__ bool strip(const Args &a, unsigned char *ring, int la
         // colour (h - 1) & 1; c0 is even and t has parity K: column q with the parity of
         constexpr int q = (K + 1) & 1;
         const N sx = q == 0 ? shup(U[h][1]) + U[h][1] : U[h][0] + shdn(U[h][0]);
-        const N nv = relax<A, CELL, KIND>(a, U[h][q], F[h][q], sx, U[h + 1][q] + U[h - 1][q], cls_of(r, c0 + q));
+        N nv = relax<A, CELL, KIND>(a, U[h][q], F[h][q], sx, U[h + 1][q] + U[h - 1][q], cls_of(r, c0 + q));
+        if constexpr (FX && OUT == kNorm)
+          if (h > S - 2) nv = stored(nv);  // the last red and the last black half-sweep
         if (rin && in(c0 + q)) U[h][q] = nv;
       }
     }
