@@ -242,6 +242,14 @@ void small2d_probe();
 bool small2d_ok(const Small2D &d);
 cudaError_t small2d_cycle(const Small2D &d, cudaStream_t s);
 
+// A cycle that starts from relative residual rho (last: the one before it) may
+// come near the FP64 rounding floor: rho is small, or no longer falls. The floor
+// of these solvers lies below 1e-14 for right-hand sides of the solution's own
+// size; above 1e-11 what a sweep's rounding adds is a thousandth of what the
+// iteration leaves, and the cheaper sweeps serve. Where the floor is higher, the
+// cycles stall and say so.
+inline bool near_floor(double rho, double last) { return rho < 1e-11 || rho > 0.7 * last; }
+
 // Sets the message mg_last_error() returns on the calling thread.
 void set_error_message(const char *msg);
 

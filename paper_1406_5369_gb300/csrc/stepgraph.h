@@ -17,7 +17,7 @@ struct StepGraphs {
     bool valid;
     unsigned key, post;
     cudaGraphExec_t exec;
-  } slot[2];
+  } slot[4];  // two live-buffer states, each with and without polished sweeps
   int next;
   cudaStream_t cap;  // private capture stream, created on first use
 };
@@ -51,7 +51,7 @@ cudaError_t step(StepGraphs &g, int k, cudaStream_t &stream, Key key, SetKey set
   cudaError_t e = cudaSuccess;
   if (!g.cap && (e = cudaStreamCreateWithFlags(&g.cap, cudaStreamNonBlocking)) != cudaSuccess) return e;
   StepGraphs::Slot &s = g.slot[g.next];
-  g.next ^= 1;
+  g.next = (g.next + 1) & 3;
   if (s.valid) cudaGraphExecDestroy(s.exec);
   s.valid = false;
   if ((e = cudaStreamBeginCapture(g.cap, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return e;
