@@ -63,6 +63,7 @@ size_t fill(const Small2D &d, int nctas, sm2::Args &a) {
   a.jacobi = d.smoother != 0;
   a.nu1 = d.nu1;
   a.nu2 = d.nu2;
+  a.polish = d.zero ? 0 : d.nu2 > 0 ? 1 : 2;  // a coarse level's correction needs no last bit
   a.zero_top = d.zero;
   a.f_top = d.f;
   a.u_top = d.u;

@@ -47,3 +47,49 @@ def test_cell_3d(n, bc, sigma, smoother, omega, nu, c):
     ref.set_rhs(f)
     ref.set_u(np.zeros_like(f))
     compare(hist, ref.solve(0.0, 40))
+
+
+# the cluster cycle: one block (up to 17, 16 cells), bands over the blocks above
+@pytest.mark.parametrize("n,smoother,omega,nu,c", [
+    (17, "rbgs", 1.0, (2, 1), (0.8, 1.3)),
+    (33, "rbgs", 1.1, (2, 2), (0.8, 1.3)),
+    (33, "jacobi", 0.8, (2, 1), (1.0, 1.0)),
+    (65, "jacobi", 0.8, (2, 2), (1.0, 1.0)),
+    (65, "rbgs", 1.0, (2, 2), (0.8, 1.3)),
+    (129, "rbgs", 1.0, (2, 1), (0.8, 1.3)),
+    (129, "jacobi", 0.8, (1, 3), (1.0, 1.0)),
+])
+def test_node_2d_cluster(n, smoother, omega, nu, c):
+    need_gpu()
+    from paper_1406_5369_gb300 import Solver
+    f = synth.uniform_rhs(2, n, 72)
+    s = Solver(2, n, smoother=smoother, omega=omega, nu1=nu[0], nu2=nu[1], stencil=c + (1.0,), maxit=40)
+    s.set_rhs(f)
+    _, _, hist = s.solve(0.0, raise_on_noconv=False)
+    ref = oracle.Hierarchy(2, n, c=c, smoother=SM[smoother], omega=omega, nu1=nu[0], nu2=nu[1])
+    ref.set_rhs(f)
+    ref.set_u(np.zeros_like(f))
+    compare(hist, ref.solve(0.0, 40))
+
+
+@pytest.mark.parametrize("n,bc,sigma,smoother,omega,nu,c", [
+    (16, "neumann", 1.0, "rbgs", 1.0, (2, 2), (1.0, 1.0)),
+    (32, "neumann", 1.0, "rbgs", 1.0, (2, 2), (1.0, 1.0)),
+    (64, "dirichlet", 1.0, "rbgs", 1.1, (2, 1), (1.0, 1.0)),
+    (64, "neumann", 500.0, "rbgs", 1.0, (2, 2), (0.9, 1.2)),
+    (128, "neumann", 1.0, "jacobi", 0.8, (2, 2), (1.0, 1.0)),
+    (128, "dirichlet", 1.0, "rbgs", 1.0, (2, 2), (1.0, 1.0)),
+])
+def test_cell_2d_cluster(n, bc, sigma, smoother, omega, nu, c):
+    need_gpu()
+    from paper_1406_5369_gb300 import CCSolver
+    f = synth.uniform(73, (n, n))
+    kw = dict(c=c, sigma=sigma, bc=bc, omega=omega, nu1=nu[0], nu2=nu[1])
+    s = CCSolver(2, n, smoother=smoother, maxit=40, **kw)
+    s.set_rhs(f)
+    s.set_solution(None)
+    _, _, hist = s.solve(0.0, raise_on_noconv=False)
+    ref = oracle.CCHierarchy(2, n, smoother=SM[smoother], **kw)
+    ref.set_rhs(f)
+    ref.set_u(np.zeros_like(f))
+    compare(hist, ref.solve(0.0, 40))
