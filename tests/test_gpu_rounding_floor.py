@@ -93,3 +93,19 @@ def test_cell_2d_cluster(n, bc, sigma, smoother, omega, nu, c):
     ref.set_rhs(f)
     ref.set_u(np.zeros_like(f))
     compare(hist, ref.solve(0.0, 40))
+
+
+@pytest.mark.parametrize("n,tau,smoother,omega,nu", [
+    (64, 1e-3, "jacobi", 0.8, (2, 2)),
+    (128, 1e-3, "rbgs", 1.1, (2, 1)),
+    (256, 1e-3, "jacobi", 0.8, (3, 2)),
+])
+def test_complex_diffusion(n, tau, smoother, omega, nu):
+    need_gpu()
+    from paper_1406_5369_gb300 import CDSolver
+    un = synth.uniform(74, (n, n)) + 0.02j * synth.uniform(75, (n, n))
+    s = CDSolver(n, tau=tau, theta=np.pi / 30, kappa=0.1, smoother=smoother, omega=omega, nu1=nu[0], nu2=nu[1], maxit=40)
+    _, _, hist = s.time_step(un, 0.0, raise_on_noconv=False)
+    ref = oracle.CDHierarchy(n, tau, np.pi / 30, 0.1, smoother=SM[smoother], omega=omega, nu1=nu[0], nu2=nu[1])
+    _, rho = ref.time_step(un, 0.0, 40)
+    compare(hist, rho)
