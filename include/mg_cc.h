@@ -84,7 +84,13 @@ mg_status mg_cc_destroy(mg_cc_ctx *ctx);
 int mg_cc_num_levels(const mg_cc_ctx *ctx);
 int mg_cc_level_size(const mg_cc_ctx *ctx, int level);
 
-/* Dense copies of a level's field: 0 = u, 1 = f, 2 = r. */
+/* Dense copies of a level's field: 0 = u, 1 = f, 2 = r. After V-cycles these are
+ * what the last cycle leaves on the level: u, f, and as r the residual after
+ * pre-smoothing. The cycles do not store all of it (small levels stay on chip,
+ * residuals are restricted as they are formed): the first call that reads or
+ * changes r of level 0 or a coarser level's field, works on a level, or takes a
+ * coarser level's norm forms the missing fields, at the cost of a cycle run
+ * operator by operator. r of level 0 is formed with the f of that moment. */
 mg_status mg_cc_set_field(mg_cc_ctx *ctx, int level, int field, const double *src);
 mg_status mg_cc_get_field(mg_cc_ctx *ctx, int level, int field, double *dst);
 

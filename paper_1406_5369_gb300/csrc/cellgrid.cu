@@ -266,10 +266,11 @@ __global__ void __launch_bounds__(kBX * kBY) kv_jacobi(const double *__restrict_
   uout[p] = gamma != 0.0 ? fma(gamma, uin[p], v) : v;
 }
 
-// Mean of the residuals of the fine cells of coarse cell x (nc per dimension).
+// Mean of the residuals of the fine cells of coarse cell x (nc per dimension);
+// uh (may be NULL) receives their values of u.
 template <int DIM>
 __device__ __forceinline__ double restricted(const double *__restrict__ u, const double *__restrict__ f, const Geo &g,
-                                             const Coef &s, const int (&x)[3], int nc) {
+                                             const Coef &s, const int (&x)[3], int nc, double *__restrict__ uh) {
   const long long st[3] = {1, g.sy, g.sz};
   const long long p = (long long)(2 * x[2]) * g.sz + (long long)(2 * x[1]) * g.sy + 2 * x[0];
   constexpr int N = 1 << DIM;
@@ -280,6 +281,7 @@ __device__ __forceinline__ double restricted(const double *__restrict__ u, const
     v[c] = u[q];
     r += f[q];
     su += v[c];
+    if (uh) uh[q] = v[c];
   }
   r = fma(-s.sigma, su, r);
 #pragma unroll
@@ -310,15 +312,15 @@ __device__ __forceinline__ double first_sweep(double f, const Coef &s, const int
   return first == 1 || (first == 2 && ((x[0] + x[1] + x[2]) & 1) == 0) ? s.wd[cls] * f : 0.0;
 }
 
-// Coarse cell: f = mean of its fine cells' residuals; u = first_sweep.
+// Coarse cell: f = mean of its fine cells' residuals; u = first_sweep. uh: see restricted.
 template <int DIM>
 __global__ void __launch_bounds__(kBX * kBY)
     kv_restrict(const double *__restrict__ u, const double *__restrict__ f, Geo g, Coef s, double *__restrict__ fc,
-                double *__restrict__ uc, Geo gc, Coef sc, int first) {
+                double *__restrict__ uc, Geo gc, Coef sc, int first, double *__restrict__ uh) {
   const int x[3] = {(int)(blockIdx.x * kBX + threadIdx.x), (int)(blockIdx.y * kBY + threadIdx.y),
                     DIM == 3 ? (int)blockIdx.z : 0};
   if (x[0] >= gc.n || x[1] >= gc.n) return;
-  const double r = restricted<DIM>(u, f, g, s, x, gc.n);
+  const double r = restricted<DIM>(u, f, g, s, x, gc.n, uh);
   const long long P = (long long)x[2] * gc.sz + (long long)x[1] * gc.sy + x[0];
   fc[P] = r;
   uc[P] = first_sweep<DIM>(r, sc, x, gc.n, first);
@@ -336,6 +338,8 @@ struct Small3 {
   const double *f, *ainv;
   double *u;
   Geo g;  // of the top level's global fields
+  double *uh, *fc;  // finest level: its pre-smoothed u and the next level's f, kept for the fields (else NULL)
+  Geo gc;
 };
 __global__ void __launch_bounds__(kSmall3Threads) kv_small3(const __grid_constant__ Small3 a) {
   __shared__ double U[2][kSmall3Lev][kSmall3Threads], F[kSmall3Lev][kSmall3Threads];
@@ -386,10 +390,12 @@ __global__ void __launch_bounds__(kSmall3Threads) kv_small3(const __grid_constan
     smooth(l, a.nu1, a.nu1 > 0 && (l > 0 || a.start >= 0), a.polish && l == 0 && a.nu2 == 0);
     if (cell(l + 1, x)) {
       const Geo g = {a.n[l], a.n[l], (long long)a.n[l] * a.n[l]};
-      const double r = restricted<3>(U[cur[l]][l], F[l], g, a.s[l], x, a.n[l + 1]);
+      const double r = restricted<3>(U[cur[l]][l], F[l], g, a.s[l], x, a.n[l + 1], nullptr);
       F[l + 1][t] = r;
       U[0][l + 1][t] = l + 2 == a.nl ? 0.0 : first_sweep<3>(r, a.s[l + 1], x, a.n[l + 1], first);
+      if (l == 0 && a.fc) a.fc[(long long)x[2] * a.gc.sz + (long long)x[1] * a.gc.sy + x[0]] = r;
     }
+    if (l == 0 && a.uh && cell(0, x)) a.uh[top] = U[cur[0]][0][t];
     __syncthreads();
   }
   {
@@ -507,6 +513,10 @@ struct mg_cc_ctx {
   double *norm_out;  // the norm (and its square)
   cudaStream_t s;
   bool polish;       // this cycle's finest level ends with sweeps in difference form
+  // The fields that a V-cycle leaves besides level 0's u (r of level 0; u, f and r
+  // of the others) are formed when a call needs them (settle): the cycle keeps the
+  // finest level's pre-smoothed u in its r, and the next level's f.
+  bool unsettled;
   mg::StepGraphs graphs;
 };
 
@@ -708,15 +718,16 @@ bool level_fx(const mg_cc_ctx *c, int l) {
   return fx_args(c, l, true, a);
 }
 
-// One pass of level l: nu (1 or 2) sweeps from the live solution (or zero) to
-// the other buffer; before them the coarse correction (corr), after them the
-// restricted residual (restr) or the partial sums of its square (nparts).
-mg_status fx_pass(mg_cc_ctx *c, int l, int nu, bool zero, bool corr, bool restr, int *nparts) {
+// One pass of level l: nu (1 or 2) sweeps from `in` (or zero) to `out`; before
+// them the coarse correction (corr), after them the restricted residual (restr)
+// or the partial sums of its square (nparts).
+mg_status fx_pass(mg_cc_ctx *c, int l, const double *in, double *out_u, int nu, bool zero, bool corr, bool restr,
+                  int *nparts) {
   Lev &L = c->lv[l], &C = c->lv[l + 1];
   mg::fx2::Args a;
   if (!fx_args(c, l, corr, a)) return ccfail(MG_EINVAL, "level %d has no fixed-point pass", l);
-  a.uin = L.u[L.cur];
-  a.uout = L.u[L.cur ^ 1];
+  a.uin = in;
+  a.uout = out_u;
   a.f = L.f;
   a.ec = corr ? C.u[C.cur] : nullptr;
   a.fc = restr ? C.f : nullptr;
@@ -728,7 +739,6 @@ mg_status fx_pass(mg_cc_ctx *c, int l, int nu, bool zero, bool corr, bool restr,
   a.pitchc = C.pitch;
   const int out = restr ? mg::fx2::kRestrict : nparts ? mg::fx2::kNorm : mg::fx2::kNone;
   CCK(mg::fx2::run(a, true, c->p.smoother != MG_RBGS, 0, nu, zero, corr, out, nparts, c->s));
-  L.cur ^= 1;
   return MG_OK;
 }
 
@@ -751,10 +761,16 @@ mg::Small2D small_desc(const mg_cc_ctx *c, int l, bool zero) {
   d.nu2 = c->p.nu2;
   d.omega = c->p.omega;
   d.zero = zero;
+  d.polish = l == 0 && c->polish;
   d.f = L.f;
   d.u = L.u[L.cur];
   d.pitch = L.pitch;
   d.dense = c->ainv;
+  if (l == 0) {
+    d.uh = L.r;
+    d.fc = c->lv[1].f;
+    d.pitchc = c->lv[1].pitch;
+  }
   return d;
 }
 
@@ -820,6 +836,11 @@ mg_status general_cycle(mg_cc_ctx *c, int l, int start) {
     a.f = L.f;
     a.u = L.u[L.cur];
     a.g = geo_of(L);
+    if (l == 0) {
+      a.uh = L.r;
+      a.fc = C.f;
+      a.gc = geo_of(C);
+    }
     a.ainv = c->ainv;
     kv_small3<<<1, kSmall3Threads, 0, c->s>>>(a);
     CCK(cudaGetLastError());
@@ -831,7 +852,7 @@ mg_status general_cycle(mg_cc_ctx *c, int l, int start) {
   const bool last = l + 2 == c->nl, own = !last && (small_desc(c, l + 1, true).lg > 0 || level_fx(c, l + 1));
   const int first = last || own || c->p.nu1 == 0 ? 0 : c->p.smoother == MG_RBGS ? 2 : 1;
   DIMCALL(c->p.dim, kv_restrict, tiles(c, C.n, C.n), dim3(kBX, kBY), L.u[L.cur], L.f, geo_of(L), coef_of(c, L), C.f,
-          C.u[C.cur], geo_of(C), coef_of(c, C), first);
+          C.u[C.cur], geo_of(C), coef_of(c, C), first, l == 0 ? L.r : nullptr);
   if (last) st = op_coarse(c);
   else if (own) st = vcycle_rec(c, l + 1, true);
   else st = general_cycle(c, l + 1, 1);
@@ -859,22 +880,23 @@ mg_status vcycle_rec(mg_cc_ctx *c, int l, bool zero, int *nparts) {
     }
   }
   if (level_fx(c, l)) {
-    // passes of at most two sweeps; more of them are passes of their own
+    // passes of at most two sweeps; more of them are passes of their own. The
+    // pre-smoothed solution goes to r, where it stays.
     int left = c->p.nu1;
     if (zero && left > 2) {
       CCK(cudaMemsetAsync(L.u[L.cur], 0, (size_t)L.count * sizeof(double), c->s));
       zero = false;
     }
-    for (; left > 2; left -= 2)
-      if ((st = fx_pass(c, l, 2, false, false, false, nullptr))) return st;
-    if ((st = fx_pass(c, l, left, zero, false, true, nullptr))) return st;
+    for (; left > 2; left -= 2, L.cur ^= 1)
+      if ((st = fx_pass(c, l, L.u[L.cur], L.u[L.cur ^ 1], 2, false, false, false, nullptr))) return st;
+    if ((st = fx_pass(c, l, L.u[L.cur], L.r, left, zero, false, true, nullptr))) return st;
     if ((st = vcycle_rec(c, l + 1, true))) return st;
     left = c->p.nu2;
     const int first = left > 2 ? 2 : left;
     left -= first;
-    if ((st = fx_pass(c, l, first, false, true, false, left ? nullptr : nparts))) return st;
-    for (; left > 0; left -= 2)
-      if ((st = fx_pass(c, l, left > 2 ? 2 : left, false, false, false, nullptr))) return st;
+    if ((st = fx_pass(c, l, L.r, L.u[L.cur], first, false, true, false, left ? nullptr : nparts))) return st;
+    for (; left > 0; left -= 2, L.cur ^= 1)
+      if ((st = fx_pass(c, l, L.u[L.cur], L.u[L.cur ^ 1], left > 2 ? 2 : left, false, false, false, nullptr))) return st;
     return MG_OK;
   }
   if (l == c->nl - 1) {
@@ -884,10 +906,39 @@ mg_status vcycle_rec(mg_cc_ctx *c, int l, bool zero, int *nparts) {
   return general_cycle(c, l, zero ? 0 : -1);
 }
 
-// The finest level runs on the kv_ kernels.
+// The finest level has sweeps in difference form (the fixed-point passes round
+// once anyway).
 bool polishes(const mg_cc_ctx *c) {
   const mg::Small2D d = small_desc(c, 0, false);
-  return !(d.lg > 0 && mg::small2d_ok(d)) && !level_fx(c, 0);
+  return (d.lg > 0 && mg::small2d_ok(d)) || !level_fx(c, 0);
+}
+
+// Algorithm 1 on level l, one operator at a time: every level keeps its u, f and r.
+mg_status plain_cycle(mg_cc_ctx *c, int l) {
+  mg_status st;
+  if (l == c->nl - 1) return op_coarse(c);
+  if ((st = op_smooth(c, l, c->p.nu1))) return st;
+  if ((st = op_residual(c, l))) return st;
+  if ((st = op_restrict(c, l))) return st;
+  Lev &C = c->lv[l + 1];
+  CCK(cudaMemsetAsync(C.u[C.cur], 0, (size_t)C.count * sizeof(double), c->s));
+  if ((st = plain_cycle(c, l + 1))) return st;
+  if ((st = op_prolong(c, l))) return st;
+  return op_smooth(c, l, c->p.nu2);
+}
+
+// Forms what the last V-cycle leaves on every level: the finest residual from the
+// pre-smoothed solution kept in r, and the coarser levels by their part of the
+// cycle, from level 1's right-hand side and zero.
+mg_status settle(mg_cc_ctx *c) {
+  if (!c->unsettled) return MG_OK;
+  c->unsettled = false;
+  Lev &L = c->lv[0], &C = c->lv[1];
+  double *uh = L.u[L.cur ^ 1];
+  CCK(cudaMemcpyAsync(uh, L.r, (size_t)L.count * sizeof(double), cudaMemcpyDeviceToDevice, c->s));
+  DIMCALL(c->p.dim, k_residual, grid_of(L, L.n), kThreads, uh, L.f, L.r, geo_of(L), coef_of(c, L));
+  CCK(cudaMemsetAsync(C.u[C.cur], 0, (size_t)C.count * sizeof(double), c->s));
+  return plain_cycle(c, 1);
 }
 
 // Step k of a solve: a V-cycle and the residual norm.
@@ -909,6 +960,7 @@ mg_status solve_step(mg_cc_ctx *c, int k) {
         return st || np == kNormDone ? st : np ? norm_final(c, np) : op_norm(c, 0);
       },
       &status));
+  c->unsettled = c->nl > 1;
   return (mg_status)status;
 }
 
@@ -999,6 +1051,7 @@ mg_status mg_cc_set_field(mg_cc_ctx *c, int level, int field, const double *src)
   if (st) return st;
   if (!src) return ccfail(MG_EINVAL, "src is NULL");
   if (field < 0 || field > 2) return ccfail(MG_EINVAL, "field must be 0 (u), 1 (f) or 2 (r)");
+  if ((level > 0 || field == 2) && (st = settle(c))) return st;
   Lev &L = c->lv[level];
   double *dst = field == 0 ? L.u[L.cur] : (field == 1 ? L.f : L.r);
   const size_t rows = (size_t)L.n * (c->p.dim == 3 ? L.n : 1);
@@ -1012,6 +1065,7 @@ mg_status mg_cc_get_field(mg_cc_ctx *c, int level, int field, double *dst) {
   if (st) return st;
   if (!dst) return ccfail(MG_EINVAL, "dst is NULL");
   if (field < 0 || field > 2) return ccfail(MG_EINVAL, "field must be 0 (u), 1 (f) or 2 (r)");
+  if ((level > 0 || field == 2) && (st = settle(c))) return st;
   Lev &L = c->lv[level];
   const double *src = field == 0 ? L.u[L.cur] : (field == 1 ? L.f : L.r);
   const size_t rows = (size_t)L.n * (c->p.dim == 3 ? L.n : 1);
@@ -1025,32 +1079,34 @@ mg_status mg_cc_smooth(mg_cc_ctx *c, int level, int sweeps) {
   mg_status st = level_ok(c, level, false);
   if (st) return st;
   if (sweeps < 0) return ccfail(MG_EINVAL, "sweeps must be >= 0");
-  return op_smooth(c, level, sweeps);
+  return (st = settle(c)) ? st : op_smooth(c, level, sweeps);
 }
 
 mg_status mg_cc_residual(mg_cc_ctx *c, int level) {
   mg_status st = level_ok(c, level, false);
-  return st ? st : op_residual(c, level);
+  return st || (st = settle(c)) ? st : op_residual(c, level);
 }
 
 mg_status mg_cc_restrict(mg_cc_ctx *c, int level) {
   mg_status st = level_ok(c, level, true);
-  return st ? st : op_restrict(c, level);
+  return st || (st = settle(c)) ? st : op_restrict(c, level);
 }
 
 mg_status mg_cc_prolongate(mg_cc_ctx *c, int level) {
   mg_status st = level_ok(c, level, true);
-  return st ? st : op_prolong(c, level);
+  return st || (st = settle(c)) ? st : op_prolong(c, level);
 }
 
 mg_status mg_cc_coarse_solve(mg_cc_ctx *c) {
   if (!c) return ccfail(MG_EINVAL, "NULL context");
-  return op_coarse(c);
+  mg_status st = settle(c);
+  return st ? st : op_coarse(c);
 }
 
 mg_status mg_cc_vcycle(mg_cc_ctx *c) {
   if (!c) return ccfail(MG_EINVAL, "NULL context");
   c->polish = polishes(c);  // how near the floor this cycle is, is not known here
+  c->unsettled = c->nl > 1;
   return vcycle_rec(c, 0);
 }
 
@@ -1058,6 +1114,7 @@ mg_status mg_cc_residual_norm(mg_cc_ctx *c, int level, double *out) {
   mg_status st = level_ok(c, level, false);
   if (st) return st;
   if (!out) return ccfail(MG_EINVAL, "out is NULL");
+  if (level > 0 && (st = settle(c))) return st;
   if ((st = op_norm(c, level))) return st;
   return read_norm(c, out);
 }

@@ -393,6 +393,7 @@ mg::Small2D small_desc(const mg_ctx *c, int l, bool zero) {
   d.nu2 = c->opt.nu2;
   d.omega = c->opt.omega;
   d.zero = zero;
+  d.polish = l == 0;  // mg_vcycle gives what a solve's steps give, so in every cycle
   d.f = (const double *)L.f;
   d.u = (double *)L.u[L.cur];
   d.pitch = L.pitch;

@@ -231,11 +231,15 @@ struct Small2D {
   int smoother, nu1, nu2;
   double omega;
   bool zero;             // start from u = 0
+  bool polish;           // the top level's last sweep in difference form (the finest level, near the rounding floor)
   const double *f;
   double *u;
   int pitch;
   const double *dense;   // coarsest inverse, NULL for a single node
   double *norm_out;      // norm of the result's residual and its square, two doubles (NULL: none)
+  // the top level's pre-smoothed u and the next level's right-hand side, for callers that keep them (NULL: not stored)
+  double *uh, *fc;
+  int pitchc;            // of fc (uh: pitch)
 };
 constexpr int kSmallTopLog = 7;  // largest level taken by default
 void small2d_probe();

@@ -63,7 +63,7 @@ size_t fill(const Small2D &d, int nctas, sm2::Args &a) {
   a.jacobi = d.smoother != 0;
   a.nu1 = d.nu1;
   a.nu2 = d.nu2;
-  a.polish = d.zero ? 0 : d.nu2 > 0 ? 1 : 2;  // a coarse level's correction needs no last bit
+  a.polish = !d.polish ? 0 : d.nu2 > 0 ? 1 : 2;
   a.zero_top = d.zero;
   a.f_top = d.f;
   a.u_top = d.u;
@@ -71,6 +71,10 @@ size_t fill(const Small2D &d, int nctas, sm2::Args &a) {
   a.kinv = 1.0 / k;
   a.k2 = k * k;
   a.norm_out = d.norm_out;
+  a.uh = d.uh;
+  a.fc = d.fc;
+  a.pitchc = d.pitchc;
+  a.kc = 0.25 * k;
   auto rows = [&](int l) { return (1 << (d.lg - l)) - (d.cell ? 0 : 1); };
   if (nd > 0) {
     const int m = rows(nd);

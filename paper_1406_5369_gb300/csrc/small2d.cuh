@@ -77,6 +77,9 @@ struct Args {
   double one;           // one node: u = f' one
   double *norm_out;     // norm of the top residual and its square (NULL: none)
   double k2;            // top k squared
+  double *uh, *fc;      // the top level's pre-smoothed u, the next level's right-hand side (NULL: not stored)
+  int pitchc;
+  double kc;            // k of the next level
   int total;            // elements of shared memory
 };
 
@@ -183,14 +186,17 @@ __device__ __forceinline__ void smooth(const Args &a, cg::cluster_group &cl, dou
 }
 
 // Residual rows of level l (node grids: the last row also to the block below).
+// uh (may be NULL): the level's solution goes there.
 template <bool CELL, bool LOCAL>
-__device__ __forceinline__ void residual(const Args &a, cg::cluster_group &cl, int l, int r, const View &x) {
+__device__ __forceinline__ void residual(const Args &a, cg::cluster_group &cl, int l, int r, const View &x, double *uh) {
   const Lev &L = a.lv[l];
+  const int off = CELL ? 1 : 0;
   double *pd = !CELL && !LOCAL && r < a.nctas - 1 ? cl.map_shared_rank(x.T, r + 1) : nullptr;
   for (int q = threadIdx.x; q < (x.R << x.lg); q += kThreads) {
     const int jl = q >> x.lg, i = (q & ((1 << x.lg) - 1)) + 1;
     if (i > x.m) continue;
     const double v = resid<CELL>(a, L, x, jl, i);
+    if (uh) uh[(long long)(x.b0 + jl - off) * a.pitch_top + i - off] = x.U[(jl + 1) * x.pitch + i];
     x.T[(jl + 1) * x.pitch + i] = v;
     if (pd && jl == x.R - 1) pd[i] = v;
   }
@@ -199,9 +205,11 @@ __device__ __forceinline__ void residual(const Args &a, cg::cluster_group &cl, i
 }
 
 // f' of the next level on rows [B0, B0 + RC): the restricted residual times 4
-// (k falls by 4 from level to level). dst row of coarse row J: (J - row0).
+// (k falls by 4 from level to level). dst row of coarse row J: (J - row0). g
+// (may be NULL): the level's global right-hand side f = f' kc.
 template <bool CELL>
-__device__ __forceinline__ void restrict_rows(const View &x, double *dst, int row0, int B0, int RC) {
+__device__ __forceinline__ void restrict_rows(const View &x, double *dst, int row0, int B0, int RC, double *g,
+                                              int pitchc, double kc) {
   const int lgc = x.lg - 1, mc = CELL ? x.m / 2 : (x.m - 1) / 2, pc = mc + 2, p = x.pitch;
   for (int q = threadIdx.x; q < (RC << lgc); q += kThreads) {
     const int J = B0 + (q >> lgc), I = (q & ((1 << lgc) - 1)) + 1;
@@ -217,6 +225,7 @@ __device__ __forceinline__ void restrict_rows(const View &x, double *dst, int ro
       v = 0.25 * fma(2.0, c, e) + t[0];
     }
     dst[(J - row0) * pc + I] = v;
+    if (g) g[(long long)(J - (CELL ? 1 : 0)) * pitchc + I - (CELL ? 1 : 0)] = v * kc;
   }
 }
 
@@ -246,9 +255,9 @@ template <bool CELL> __device__ __forceinline__ void local_cycle(const Args &a, 
   for (int l = first; l < last; l++) {
     View x = view(a, sm, l, 0);
     smooth<CELL, true>(a, cl, sm, l, 0, x, a.nu1, l == 0 && a.polish == 2);
-    residual<CELL, true>(a, cl, l, 0, x);
+    residual<CELL, true>(a, cl, l, 0, x, l == 0 ? a.uh : nullptr);
     const View c = view(a, sm, l + 1, 0);
-    restrict_rows<CELL>(x, c.F, 1, 1, c.R);
+    restrict_rows<CELL>(x, c.F, 1, 1, c.R, l == 0 ? a.fc : nullptr, a.pitchc, a.kc);
     __syncthreads();
   }
   {
@@ -307,11 +316,12 @@ template <bool CELL> __global__ void __launch_bounds__(kThreads, 1) k_small2d(co
   for (int l = 0; l < a.nd; l++) {
     View x = view(a, sm, l, r);
     smooth<CELL, false>(a, cl, sm, l, r, x, a.nu1, l == 0 && a.polish == 2);
-    residual<CELL, false>(a, cl, l, r, x);
+    residual<CELL, false>(a, cl, l, r, x, l == 0 ? a.uh : nullptr);
     const int B0 = a.band[l + 1][r], RC = a.band[l + 1][r + 1] - B0;
     double *G = sm + a.lv[l + 1].f;
-    if (l + 1 < a.nd) restrict_rows<CELL>(x, G, B0, B0, RC);
-    else restrict_rows<CELL>(x, cl.map_shared_rank(G, 0), 1, B0, RC);
+    double *g = l == 0 ? a.fc : nullptr;
+    if (l + 1 < a.nd) restrict_rows<CELL>(x, G, B0, B0, RC, g, a.pitchc, a.kc);
+    else restrict_rows<CELL>(x, cl.map_shared_rank(G, 0), 1, B0, RC, g, a.pitchc, a.kc);
     __syncthreads();
   }
   if (a.nd > 0) cl.sync();

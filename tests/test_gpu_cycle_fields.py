@@ -1,0 +1,102 @@
+"""The fields that V-cycles leave on every level (u, f and r, the residual after
+pre-smoothing) are those of Algorithm 1 run one operator at a time, whichever
+kernels the cycle took, and reading them changes nothing.
+
+Tolerances: u to 1e-12 of the finest one (which it corrects), f of a coarse level
+and r, which are differences, to 1e-12 of diag times the largest u of the level
+they come from: some thousand times the rounding of the few dozen operations
+behind each value.
+The coarse fields have to be of the finest one's order for that: one cycle from a
+random start, or three with sweeps weak enough (omega = 0.3) to leave an error.
+"""
+import numpy as np
+import pytest
+
+import synth
+from gpu_util import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def plain_cycle(s, nu1, nu2, l=0, zero=None):
+    """Algorithm 1 by the level operators."""
+    if l == s.levels - 1:
+        s.coarse_solve()
+        return
+    s.smooth(l, nu1)
+    s.residual(l)
+    s.restrict(l)
+    s.set_field(l + 1, "u", np.zeros_like(s.get_field(l + 1, "u")))
+    plain_cycle(s, nu1, nu2, l + 1)
+    s.prolongate(l)
+    s.smooth(l, nu2)
+
+
+def compare(s, ref, diag, order):
+    top = s.get_field(0, "u")
+    for l, name in order:
+        got, want = s.get_field(l, name), ref.get_field(l, name)
+        scale = np.abs(ref.get_field(0, "u")).max()
+        if name != "u":
+            scale = max(diag(max(l - 1, 0)) * np.abs(ref.get_field(max(l - 1, 0), "u")).max(), np.abs(want).max())
+        assert np.abs(got - want).max() <= 1e-12 * scale, (l, name)
+    assert np.array_equal(s.get_field(0, "u"), top)
+
+
+def every(levels):
+    """r of a middle level first, then everything."""
+    return [(levels // 2, "r")] + [(l, name) for l in range(levels) for name in ("r", "f", "u")]
+
+
+@pytest.mark.parametrize("dim,n,bc,smoother,omega,nu,nc", [
+    (2, 8, "neumann", "rbgs", 1.0, (2, 1), 1),
+    (2, 64, "neumann", "jacobi", 0.8, (2, 1), 2),
+    (2, 128, "dirichlet", "rbgs", 1.1, (2, 2), 1),
+    (2, 128, "neumann", "rbgs", 1.0, (0, 2), 4),
+    (2, 512, "neumann", "rbgs", 1.0, (2, 2), 1),
+    (2, 256, "dirichlet", "jacobi", 0.8, (3, 3), 2),
+    (2, 256, "neumann", "rbgs", 1.0, (2, 0), 1),
+    (3, 4, "dirichlet", "rbgs", 1.0, (2, 2), 2),
+    (3, 8, "neumann", "jacobi", 0.8, (1, 2), 1),
+    (3, 32, "neumann", "rbgs", 1.0, (2, 2), 1),
+    (3, 64, "dirichlet", "jacobi", 0.8, (0, 3), 4),
+    (3, 64, "dirichlet", "rbgs", 1.2, (3, 0), 1),
+])
+@pytest.mark.parametrize("solve", [False, True])
+def test_cell_centred(dim, n, bc, smoother, omega, nu, nc, solve):
+    need_gpu()
+    from paper_1406_5369_gb300 import CCSolver
+    f, u0 = synth.uniform(81, (n,) * dim), synth.uniform(82, (n,) * dim)
+    kw = dict(sigma=3.0, bc=bc, smoother=smoother, omega=0.3 if solve else omega, nu1=nu[0], nu2=nu[1], coarsest_n=nc,
+              maxit=3)
+    s, ref = CCSolver(dim, n, **kw), CCSolver(dim, n, **kw)
+    for t in (s, ref):
+        t.set_rhs(f)
+        t.set_solution(u0)
+    if solve:  # three steps, the last one a replayed graph
+        s.solve(0.0, raise_on_noconv=False)
+    else:
+        s.vcycle()
+    for _ in range(3 if solve else 1):
+        plain_cycle(ref, *nu)
+    compare(s, ref, lambda l: 4.0 * dim * (n >> l) ** 2, every(s.levels))
+
+
+def test_cell_centred_level_calls_after_a_cycle():
+    """Level operators and norms work on the fields that the cycle leaves."""
+    need_gpu()
+    from paper_1406_5369_gb300 import CCSolver
+    n = 256
+    f = synth.uniform(83, (n, n))
+    for call in (lambda t: t.restrict(0), lambda t: t.prolongate(1), lambda t: t.smooth(2, 1), lambda t: t.residual(3),
+                 lambda t: t.set_field(2, "u", np.ones((n // 4, n // 4))), lambda t: t.coarse_solve()):
+        s, ref = CCSolver(2, n), CCSolver(2, n)
+        for t in (s, ref):
+            t.set_rhs(f)
+            t.set_solution(None)
+        s.vcycle()
+        plain_cycle(ref, 2, 1)
+        call(s)
+        call(ref)
+        compare(s, ref, lambda l: 8.0 * (n >> l) ** 2, every(s.levels))
+        assert abs(s.residual_norm(2) - ref.residual_norm(2)) <= 1e-10 * ref.residual_norm(0)
