@@ -304,16 +304,23 @@ __global__ void __launch_bounds__(kBX * kBY) kr_rbgs_half(double2 *u, const doub
 
 // Coarse cell (I, J): f = mean of the four residuals, g = wd f, and u after the
 // first sweep (Jacobi: g) or red half-sweep from zero; u = 0 when there is no
-// pre-smoothing (first = 0: none, 1: Jacobi, 2: red-black).
+// pre-smoothing (first = 0: none, 1: Jacobi, 2: red-black). uh (may be NULL)
+// receives the fine u.
 __global__ void __launch_bounds__(kBX * kBY)
     kr_restrict(const double2 *__restrict__ u, const double2 *__restrict__ f, const double2 *__restrict__ w, Geo g,
                 Ph ph, double2 *__restrict__ fc, double2 *__restrict__ gfc, double2 *__restrict__ uc,
-                const double2 *__restrict__ wdc, Geo gc, int first) {
+                const double2 *__restrict__ wdc, Geo gc, int first, double2 *__restrict__ uh) {
   int I, J;
   if (!cell(gc.n, I, J)) return;
   const int i = 2 * I, j = 2 * J;
   const long long p = (long long)j * g.sy + i, sy = g.sy;
   const double2 a = u[p], b = u[p + 1], c = u[p + sy], d = u[p + sy + 1];
+  if (uh) {
+    uh[p] = a;
+    uh[p + 1] = b;
+    uh[p + sy] = c;
+    uh[p + sy + 1] = d;
+  }
   double2 s = make_double2(0.0, 0.0);
   if (i > 0) {
     face_add(s, w[p - 1].x, csub(a, u[p - 1]));
@@ -383,7 +390,16 @@ __global__ void __launch_bounds__(kBX * kBY) kr_diag(const double2 *__restrict__
   q[p] = cmul(d, make_double2(ph.x, ph.y));
   if (f) gf[p] = cmul(d, f[p]);
 }
-// The complex faces from the weights, in place: gx holds w on entry.
+// The complex x-faces (y: y-faces) from the weights.
+__global__ void __launch_bounds__(kBX * kBY) kr_face(const double2 *__restrict__ w, double2 *__restrict__ out, Geo g,
+                                                     double er, double ei, int y) {
+  int i, j;
+  if (!cell(g.n, i, j)) return;
+  const long long p = (long long)j * g.sy + i;
+  const double v = y ? w[p].y : w[p].x;
+  out[p] = make_double2(er * v, ei * v);
+}
+// The same, both, in place: gx holds w on entry.
 __global__ void __launch_bounds__(kBX * kBY) kr_expand(double2 *gx, double2 *__restrict__ gy, Geo g, double er,
                                                        double ei) {
   int i, j;
@@ -430,9 +446,12 @@ struct mg_cd_ctx {
   double *partials, *norm_out;
   cudaStream_t s;
   // The faces are e^{i theta} times real weights (set by begin_step): V-cycles
-  // run on the kr_ kernels. A call that sets or reads faces, sets f or r, reads r
-  // or works on one level first expands the faces (to_complex).
+  // run on the kr_ kernels. A call that sets faces, f, r or a coarse u, reads r or
+  // works on one level first expands the faces (to_complex).
   bool phased;
+  // A phased cycle has run: its finest pre-smoothed u is in level 0's wd, which
+  // these cycles do not need, and r is still to be formed (to_complex).
+  bool unsettled;
   bool polish;  // this cycle's finest level ends with sweeps in difference form
   mg::StepGraphs graphs;
 };
@@ -588,17 +607,6 @@ dim3 tiles(int nx, int ny) { return dim3((unsigned)((nx + kBX - 1) / kBX), (unsi
     CDK(cudaGetLastError());                                       \
   } while (0)
 
-// Phased faces back to complex ones on every level.
-mg_status to_complex(mg_cd_ctx *c) {
-  if (!c->phased) return MG_OK;
-  for (int l = 0; l < c->nl; l++) {
-    Lev &L = c->lv[l];
-    LAUNCH2(kr_expand, L.n, L.n, L.gx, L.gy, geo_of(L), cos(c->p.theta), sin(c->p.theta));
-  }
-  c->phased = false;
-  return MG_OK;
-}
-
 // Sweeps of level l with phased faces; skip: the first sweep (Jacobi) or red
 // half-sweep is already in u; polish: in difference form.
 mg_status phased_smooth(mg_cd_ctx *c, int l, int sweeps, bool skip, bool polish) {
@@ -633,7 +641,7 @@ mg_status phased_cycle(mg_cd_ctx *c, int l, bool begun) {
   Lev &L = c->lv[l], &C = c->lv[l + 1];
   if ((st = phased_smooth(c, l, c->p.nu1, begun && c->p.nu1 > 0, c->polish && l == 0 && c->p.nu2 == 0))) return st;
   LAUNCH2(kr_restrict, C.n, C.n, L.u[L.cur], L.f, L.gx, geo_of(L), phase_of(c, L), C.f, C.gf, C.u[C.cur], C.wd,
-          geo_of(C), c->p.nu1 == 0 ? 0 : c->p.smoother == MG_RBGS ? 2 : 1);
+          geo_of(C), c->p.nu1 == 0 ? 0 : c->p.smoother == MG_RBGS ? 2 : 1, l == 0 ? L.wd : nullptr);
   if ((st = phased_cycle(c, l + 1, true))) return st;
   if ((st = op_prolong(c, l))) return st;
   return phased_smooth(c, l, c->p.nu2, false, c->polish && l == 0);
@@ -653,9 +661,42 @@ mg_status vcycle_rec(mg_cd_ctx *c, int l) {
   return op_smooth(c, l, c->p.nu2);
 }
 
+mg_status op_wdiag(mg_cd_ctx *c, int l) {
+  Lev &L = c->lv[l];
+  LAUNCH(k_wdiag, grid_of(L, L.n), L.gx, L.gy, L.wd, geo_of(L), s_of(c, L), c->p.omega);
+  return MG_OK;
+}
+
+// Phased faces back to complex ones on every level, and the fields as a cycle on
+// those leaves them: r of level 0 from the pre-smoothed u, the coarser levels by
+// their part of the cycle, from level 1's right-hand side and zero. Without a
+// cycle r is the residual of what the levels hold.
+mg_status to_complex(mg_cd_ctx *c) {
+  if (!c->phased) return MG_OK;
+  for (int l = 0; l < c->nl; l++) {
+    Lev &L = c->lv[l];
+    LAUNCH2(kr_expand, L.n, L.n, L.gx, L.gy, geo_of(L), cos(c->p.theta), sin(c->p.theta));
+  }
+  c->phased = false;
+  mg_status st;
+  if (!c->unsettled) {
+    for (int l = 0; l < c->nl; l++)
+      if ((st = op_residual(c, l))) return st;
+    return MG_OK;
+  }
+  c->unsettled = false;
+  Lev &L = c->lv[0], &C = c->lv[1];
+  LAUNCH(k_residual, grid_of(L, L.n), L.wd, L.f, L.r, L.gx, L.gy, geo_of(L), s_of(c, L));
+  if ((st = op_wdiag(c, 0))) return st;
+  CDK(cudaMemsetAsync(C.u[C.cur], 0, (size_t)C.count * sizeof(double2), c->s));
+  if ((st = vcycle_rec(c, 1))) return st;
+  return op_residual(c, c->nl - 1);  // no cycle writes the coarsest r: zero, its system is solved
+}
+
 // Step k of a solve: a V-cycle and the residual norm.
 mg_status solve_step(mg_cd_ctx *c, int k) {
   int status = 0;
+  c->unsettled = c->phased && c->nl > 1;
   CDK(mg::step(
       c->graphs, k, c->s,
       [&] {
@@ -689,12 +730,6 @@ double2 *field_ptr(Lev &L, int field) {
     case MG_CD_GY: return L.gy;
     default: return nullptr;
   }
-}
-
-mg_status op_wdiag(mg_cd_ctx *c, int l) {
-  Lev &L = c->lv[l];
-  LAUNCH(k_wdiag, grid_of(L, L.n), L.gx, L.gy, L.wd, geo_of(L), s_of(c, L), c->p.omega);
-  return MG_OK;
 }
 
 mg_status copy_in(mg_cd_ctx *c, Lev &L, double2 *dst, const double *src) {
@@ -775,7 +810,7 @@ mg_status mg_cd_set_field(mg_cd_ctx *c, int level, int field, const double *src)
   if (!src) return cdfail(MG_EINVAL, "src is NULL");
   double2 *dst = field_ptr(c->lv[level], field);
   if (!dst) return cdfail(MG_EINVAL, "unknown field %d", field);
-  if (field != MG_CD_U && (st = to_complex(c))) return st;
+  if ((field != MG_CD_U || level > 0) && (st = to_complex(c))) return st;
   if ((st = copy_in(c, c->lv[level], dst, src))) return st;
   return (field == MG_CD_GX || field == MG_CD_GY) ? op_wdiag(c, level) : MG_OK;
 }
@@ -787,8 +822,11 @@ mg_status mg_cd_get_field(mg_cd_ctx *c, int level, int field, double *dst) {
   Lev &L = c->lv[level];
   const double2 *src = field_ptr(L, field);
   if (!src) return cdfail(MG_EINVAL, "unknown field %d", field);
-  if (field == MG_CD_R && c->phased && ((st = to_complex(c)) || (st = op_residual(c, level)))) return st;
-  if ((field == MG_CD_GX || field == MG_CD_GY) && (st = to_complex(c))) return st;
+  if (field == MG_CD_R && (st = to_complex(c))) return st;
+  if ((field == MG_CD_GX || field == MG_CD_GY) && c->phased) {
+    LAUNCH2(kr_face, L.n, L.n, L.gx, L.u[L.cur ^ 1], geo_of(L), cos(c->p.theta), sin(c->p.theta), field == MG_CD_GY);
+    src = L.u[L.cur ^ 1];
+  }
   CDK(cudaMemcpy2DAsync(dst, (size_t)L.n * 16, src, (size_t)L.pitch * 16, (size_t)L.n * 16, (size_t)L.n,
                         cudaMemcpyDefault, c->s));
   CDK(cudaStreamSynchronize(c->s));
@@ -814,6 +852,7 @@ mg_status mg_cd_begin_step(mg_cd_ctx *c, const double *un) {
     LAUNCH2(kr_diag, F.n, F.n, F.gx, geo_of(F), phase_of(c, F), c->p.omega, F.wd, F.gy, l == 0 ? F.f : nullptr, F.gf);
   }
   c->phased = true;
+  c->unsettled = false;
   // where 1 / s would overflow (A is the identity there), or s, the complex faces serve
   const double s0 = s_of(c, L);
   return s0 > 1e-100 && s0 < 1e100 ? MG_OK : to_complex(c);
@@ -850,6 +889,7 @@ mg_status mg_cd_coarse_solve(mg_cd_ctx *c) {
 mg_status mg_cd_vcycle(mg_cd_ctx *c) {
   if (!c) return cdfail(MG_EINVAL, "NULL context");
   c->polish = true;  // how near the floor this cycle is, is not known here
+  c->unsettled = c->phased && c->nl > 1;
   return vcycle_rec(c, 0);
 }
 
@@ -857,7 +897,6 @@ mg_status mg_cd_residual_norm(mg_cd_ctx *c, int level, double *out) {
   mg_status st = level_ok(c, level, false);
   if (st) return st;
   if (!out) return cdfail(MG_EINVAL, "out is NULL");
-  if (level != 0 && (st = to_complex(c))) return st;
   if ((st = op_norm(c, level))) return st;
   return read_norm(c, out);
 }

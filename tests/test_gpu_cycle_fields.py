@@ -100,3 +100,65 @@ def test_cell_centred_level_calls_after_a_cycle():
         call(ref)
         compare(s, ref, lambda l: 8.0 * (n >> l) ** 2, every(s.levels))
         assert abs(s.residual_norm(2) - ref.residual_norm(2)) <= 1e-10 * ref.residual_norm(0)
+
+
+def cd_pair(n, **kw):
+    need_gpu()
+    from paper_1406_5369_gb300 import CDSolver
+    un = synth.uniform(84, (n, n)) + 0.05j * synth.uniform(85, (n, n))
+    s, ref = CDSolver(n, tau=1e-2, **kw), CDSolver(n, tau=1e-2, **kw)
+    for t in (s, ref):
+        t.begin_step(un)
+    return s, ref
+
+
+@pytest.mark.parametrize("n,smoother,omega,nu", [
+    (2, "rbgs", 1.0, (2, 2)),
+    (64, "rbgs", 1.0, (2, 2)),
+    (128, "jacobi", 0.8, (2, 1)),
+    (256, "jacobi", 0.8, (0, 2)),
+    (256, "rbgs", 1.2, (3, 0)),
+])
+@pytest.mark.parametrize("solve", [False, True])
+@pytest.mark.parametrize("face_first", [False, True])
+def test_complex_diffusion(n, smoother, omega, nu, solve, face_first):
+    s, ref = cd_pair(n, smoother=smoother, omega=0.3 if solve else omega, nu1=nu[0], nu2=nu[1], maxit=3)
+    if solve:
+        s.solve(0.0, raise_on_noconv=False)
+    else:
+        s.vcycle()
+    for _ in range(3 if solve else 1):
+        plain_cycle(ref, *nu)
+    if face_first:
+        assert np.array_equal(s.get_field(0, "gx"), ref.get_field(0, "gx"))
+    compare(s, ref, lambda l: 1.0 + 4e-2 * (n >> l) ** 2, every(s.levels))
+
+
+def test_complex_diffusion_faces_and_norms_leave_the_cycles_as_they_are():
+    s, ref = cd_pair(128)
+    for t in (s, ref):
+        t.vcycle()
+    for l in range(s.levels):
+        for name in ("gx", "gy"):
+            s.get_field(l, name)
+        s.residual_norm(l)
+    for t in (s, ref):
+        t.vcycle()
+    assert np.array_equal(s.get_field(0, "u"), ref.get_field(0, "u"))  # the same kernels still
+    # the faces are the same on either kind of context, and so are the norms
+    norms = [s.residual_norm(l) for l in range(s.levels)]
+    faces = [s.get_field(l, name) for l in range(s.levels) for name in ("gx", "gy")]
+    s.residual(0)
+    assert all(abs(s.residual_norm(l) - v) <= 1e-12 * norms[0] for l, v in enumerate(norms))
+    assert all(np.array_equal(a, s.get_field(l, name))
+               for a, (l, name) in zip(faces, [(l, name) for l in range(s.levels) for name in ("gx", "gy")]))
+
+
+def test_complex_diffusion_residual_before_any_cycle():
+    s, ref = cd_pair(64)
+    ref.residual(0)
+    r = s.get_field(0, "r")
+    assert np.abs(r - ref.get_field(0, "r")).max() <= 1e-13 * 170
+    s.restrict(0)
+    ref.restrict(0)
+    assert np.abs(s.get_field(1, "f") - ref.get_field(1, "f")).max() <= 1e-13 * 170
