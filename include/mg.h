@@ -222,7 +222,16 @@ mg_status mg_get_solution(mg_ctx *ctx, double *u);
 /* Per-level access used by operator-level tests and tools: level ell's
  * solution U, right-hand side F or residual R, as dense n_ell^dim FP64
  * (converted from/to the level's storage type). In the *_DC precisions
- * the levels are the inner hierarchy (U = correction e, F = defect d). */
+ * the levels are the inner hierarchy (U = correction e, F = defect d).
+ * A V-cycle leaves U, F and R of every level with fuse = 0. With fuse = 1 it
+ * leaves no R where smoothing, residual and restriction are one kernel (2D,
+ * red-black), and no coarser field below a level that one block or one cluster
+ * takes with everything under it (2D: 65 in *_DC precisions, cluster_max_n; FP64:
+ * 33; 3D: 17, FP64 9). Larger FP64 levels that the cluster or the fixed-point
+ * passes take do leave theirs: the first call that reads or changes R of level 0
+ * or a coarser level's field, works on a level, takes a coarser level's norm or
+ * adds the context to a batch forms them, at the cost of a cycle's coarser levels.
+ * R of level 0 is formed with the F of that moment. */
 mg_status mg_set_field(mg_ctx *ctx, int level, mg_field field, const double *src);
 mg_status mg_get_field(mg_ctx *ctx, int level, mg_field field, double *dst);
 

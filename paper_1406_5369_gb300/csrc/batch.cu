@@ -1456,6 +1456,7 @@ mg_status mg_batch_add(mg_batch *b, mg_ctx *c, int *id) {
         b->fp64 = !c->dc;
         b->have_opts = true;
       }
+      if (mg_status st = mg::settle(c)) return st;  // the batch works on the same fields
       // the batch's kernels read what the context's stream wrote (its
       // right-hand side, a reset solution): order them after it
       if (c->stream != b->stream &&

@@ -49,11 +49,23 @@ struct GraphSlot {
   int pairs[kSlotPairs];
 };
 
+struct mg_ctx;
+namespace mg {
+// Forms the fields that the last V-cycle has yet to leave.
+mg_status settle(mg_ctx *c);
+}  // namespace mg
+
 struct mg_ctx {
   int dim, n, nl;
   int variable;
   bool dc;                // defect-correction precision
   bool bc_zero;           // homogeneous Dirichlet data
+  // FP64 cycles on the cluster or the fixed-point passes leave the coarser levels'
+  // u and f, and r where cycles of one kernel per operator form it, to settle():
+  // the next level's right-hand side is kept, and (uh_in_r) the finest level's
+  // pre-smoothed u in its r.
+  bool unsettled, uh_in_r;
+  bool replay;            // settle() is running the coarser levels: not on those kernels
   bool u_zero;            // the finest (user-level) interior solution is known to be zero
   mg_options opt;
   cudaStream_t stream;    // user stream

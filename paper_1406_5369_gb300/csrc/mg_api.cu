@@ -353,27 +353,30 @@ bool level_fused(mg_ctx *c, int l) {
 // keeps the block-tile kernels up to it.
 bool level_fx(const mg_ctx *c, int l) {
   const Level &L = c->lv[l];
-  return c->opt.fuse && !c->dc && l + 1 < c->nl && c->opt.nu1 >= 1 && c->opt.nu2 >= 1 &&
+  return c->opt.fuse && !c->dc && !c->replay && l + 1 < c->nl && c->opt.nu1 >= 1 && c->opt.nu2 >= 1 &&
          L.n > c->opt.tile_max_n && L.n > mg::coarse_top_n(c->dim, true) && c->opt.fuse_depth == 0 &&
          c->lv[l + 1].dtype == mg::F64 && mg::d2::fx_ok(L, (int)c->opt.smoother, c->opt.omega);
 }
 
 // True when level l runs on the fixed-point 3D passes (fx3d.cuh).
 bool level_fx3(const mg_ctx *c, int l) {
-  return c->opt.fuse && !c->dc && c->dim == 3 && l + 1 < c->nl && c->opt.nu1 >= 1 && c->opt.nu2 >= 1 &&
+  return c->opt.fuse && !c->dc && !c->replay && c->dim == 3 && l + 1 < c->nl && c->opt.nu1 >= 1 && c->opt.nu2 >= 1 &&
          c->lv[l + 1].dtype == mg::F64 && mg::d3::fx_ok(c->lv[l], (int)c->opt.smoother, c->opt.omega);
 }
 
-// One fixed-point pass (one sweep) of level l from the live solution buffer to the other.
-mg_status fx3_pass(mg_ctx *c, int l, int kind, bool zero, bool corr, bool restr, int *nparts, cudaStream_t s) {
+// One fixed-point pass (one sweep) of level l from `in` to `out`.
+mg_status fx3_pass(mg_ctx *c, int l, int kind, void *in, void *out, bool zero, bool corr, bool restr, int *nparts,
+                   cudaStream_t s) {
   Level &L = c->lv[l], &C = c->lv[l + 1];
   TLAUNCH(c, kind, l, s,
-          mg::d3::fx_pass(L, &C, (int)c->opt.smoother, c->opt.omega, L.u[L.cur], L.u[L.cur ^ 1], zero,
-                          corr ? C.u[C.cur] : nullptr, restr ? C.f : nullptr, nparts ? c->partials : nullptr, nparts,
-                          s));
-  L.cur ^= 1;
+          mg::d3::fx_pass(L, &C, (int)c->opt.smoother, c->opt.omega, in, out, zero, corr ? C.u[C.cur] : nullptr,
+                          restr ? C.f : nullptr, nparts ? c->partials : nullptr, nparts, s));
   return MG_OK;
 }
+
+// A cycle of one kernel per operator forms r (the fused red-black 2D passes do
+// not, and leave what is there): the pre-smoothed solution goes to r, where it stays.
+bool keeps_uh(const mg_ctx *c) { return c->dim == 3 || c->opt.smoother == MG_JACOBI; }
 
 // The cluster V-cycle of levels l .. nl-1 (small2d.cuh); lg = 0 when the
 // context or the level does not take it. cluster_max_n sets its largest level.
@@ -382,7 +385,7 @@ mg::Small2D small_desc(const mg_ctx *c, int l, bool zero) {
   memset(&d, 0, sizeof d);
   const Level &L = c->lv[l];
   const int top = c->opt.cluster_max_n > 0 ? c->opt.cluster_max_n : (1 << mg::kSmallTopLog) + 1;
-  if (!c->opt.fuse || c->dc || c->dim != 2 || c->variable || L.n > top || l + 1 >= c->nl) return d;
+  if (!c->opt.fuse || c->dc || c->replay || c->dim != 2 || c->variable || L.n > top || l + 1 >= c->nl) return d;
   while ((1 << d.lg) + 1 < L.n) d.lg++;
   d.nlev = c->nl - l;
   d.kx = L.c[0] * L.inv_h2;
@@ -398,17 +401,29 @@ mg::Small2D small_desc(const mg_ctx *c, int l, bool zero) {
   d.u = (double *)L.u[L.cur];
   d.pitch = L.pitch;
   d.dense = c->lv[c->nl - 1].dense;
+  if (l == 0) {
+    d.uh = keeps_uh(c) ? (double *)L.r : nullptr;
+    d.fc = (double *)c->lv[1].f;
+    d.pitchc = c->lv[1].pitch;
+  }
   return d;
 }
 
-// One fixed-point pass of level l (mg::d2::fx_pass) from the live solution buffer to the other.
-mg_status fx_pass(mg_ctx *c, int l, int kind, int nu, bool zero, bool corr, bool restr, int *nparts, cudaStream_t s) {
+// Level 0 runs on the cluster or the fixed-point passes, where it had kernels
+// that leave the fields of the coarser levels.
+bool leaves_later(mg_ctx *c) {
+  if (c->dc || c->nl < 2 || c->lv[0].n <= mg::coarse_top_n(c->dim, true)) return false;
+  const mg::Small2D d = small_desc(c, 0, false);
+  return (d.lg > 0 && mg::small2d_ok(d)) || level_fx(c, 0) || level_fx3(c, 0);
+}
+
+// One fixed-point pass of level l (mg::d2::fx_pass) from `in` to `out`.
+mg_status fx_pass(mg_ctx *c, int l, int kind, void *in, void *out, int nu, bool zero, bool corr, bool restr,
+                  int *nparts, cudaStream_t s) {
   Level &L = c->lv[l], &C = c->lv[l + 1];
   TLAUNCH(c, kind, l, s,
-          mg::d2::fx_pass(L, &C, (int)c->opt.smoother, c->opt.omega, nu, L.u[L.cur], L.u[L.cur ^ 1], zero,
-                          corr ? C.u[C.cur] : nullptr, restr ? C.f : nullptr, nparts ? c->partials : nullptr, nparts,
-                          c->opt.tile_rows, s));
-  L.cur ^= 1;
+          mg::d2::fx_pass(L, &C, (int)c->opt.smoother, c->opt.omega, nu, in, out, zero, corr ? C.u[C.cur] : nullptr,
+                          restr ? C.f : nullptr, nparts ? c->partials : nullptr, nparts, c->opt.tile_rows, s));
   return MG_OK;
 }
 
@@ -458,25 +473,38 @@ mg_status vcycle_rec(mg_ctx *c, int l, bool zero, cudaStream_t s, int *nparts = 
       if ((st = op_zero_u(c, l, s))) return st;
       zero = false;
     }
-    for (; left > 2; left -= 2)
-      if ((st = fx_pass(c, l, MG_KERNEL_PRESMOOTH, 2, false, false, false, nullptr, s))) return st;
-    if ((st = fx_pass(c, l, MG_KERNEL_PRESMOOTH, left, zero, false, true, nullptr, s))) return st;
+    for (; left > 2; left -= 2, L.cur ^= 1)
+      if ((st = fx_pass(c, l, MG_KERNEL_PRESMOOTH, L.u[L.cur], L.u[L.cur ^ 1], 2, false, false, false, nullptr, s)))
+        return st;
+    void *uh = keeps_uh(c) ? L.r : L.u[L.cur ^ 1];
+    if ((st = fx_pass(c, l, MG_KERNEL_PRESMOOTH, L.u[L.cur], uh, left, zero, false, true, nullptr, s))) return st;
     if ((st = vcycle_rec(c, l + 1, true, s))) return st;
     left = c->opt.nu2;
     const int first = left > 2 ? 2 : left;
     left -= first;
-    if ((st = fx_pass(c, l, MG_KERNEL_POSTSMOOTH, first, false, true, false, left ? nullptr : nparts, s))) return st;
-    for (; left > 0; left -= 2)
-      if ((st = fx_pass(c, l, MG_KERNEL_POSTSMOOTH, left > 2 ? 2 : left, false, false, false, nullptr, s))) return st;
+    if ((st = fx_pass(c, l, MG_KERNEL_POSTSMOOTH, uh, L.u[L.cur], first, false, true, false, left ? nullptr : nparts, s)))
+      return st;
+    for (; left > 0; left -= 2, L.cur ^= 1)
+      if ((st = fx_pass(c, l, MG_KERNEL_POSTSMOOTH, L.u[L.cur], L.u[L.cur ^ 1], left > 2 ? 2 : left, false, false, false,
+                        nullptr, s)))
+        return st;
     return MG_OK;
   }
   if (level_fx3(c, l)) {
-    for (int k = 0; k < c->opt.nu1; k++)
-      if ((st = fx3_pass(c, l, MG_KERNEL_PRESMOOTH, zero && k == 0, false, k + 1 == c->opt.nu1, nullptr, s))) return st;
-    if ((st = vcycle_rec(c, l + 1, true, s))) return st;
-    for (int k = 0; k < c->opt.nu2; k++)
-      if ((st = fx3_pass(c, l, MG_KERNEL_POSTSMOOTH, false, k == 0, false, k + 1 == c->opt.nu2 ? nparts : nullptr, s)))
+    for (int k = 0; k < c->opt.nu1; k++) {
+      const bool end = k + 1 == c->opt.nu1;
+      if ((st = fx3_pass(c, l, MG_KERNEL_PRESMOOTH, L.u[L.cur], end ? L.r : L.u[L.cur ^ 1], zero && k == 0, false, end,
+                         nullptr, s)))
         return st;
+      if (!end) L.cur ^= 1;
+    }
+    if ((st = vcycle_rec(c, l + 1, true, s))) return st;
+    for (int k = 0; k < c->opt.nu2; k++) {
+      if ((st = fx3_pass(c, l, MG_KERNEL_POSTSMOOTH, k == 0 ? L.r : L.u[L.cur], k == 0 ? L.u[L.cur] : L.u[L.cur ^ 1],
+                         false, k == 0, false, k + 1 == c->opt.nu2 ? nparts : nullptr, s)))
+        return st;
+      if (k > 0) L.cur ^= 1;
+    }
     return MG_OK;
   }
   if (level_fused(c, l)) {
@@ -691,6 +719,8 @@ void drop_graphs(mg_ctx *c) {
 // the state it leaves behind (Jacobi sweeps flip a level's live buffer).
 mg_status run(mg_ctx *c, int kind) {
   NvtxRange range(kind ? "mg solve step" : "mg V-cycle");
+  c->unsettled = leaves_later(c);
+  c->uh_in_r = c->unsettled && keeps_uh(c);
   if (!c->opt.use_graph) return record(c, kind, c->stream);
   unsigned key = cur_key(c);
   for (int i = 0; i < kGraphSlots; i++) {
@@ -756,6 +786,34 @@ mg_status read_norm(mg_ctx *c, double *out) {
 }
 
 }  // namespace
+
+namespace mg {
+mg_status settle(mg_ctx *c) {
+  if (!c->unsettled) return MG_OK;
+  c->unsettled = false;
+  Level &L = c->lv[0];
+  mg_status st;
+  if (c->uh_in_r) {
+    // inner nodes only: the buffer's boundary nodes hold the Dirichlet values
+    void *uh = L.u[L.cur ^ 1];
+    const size_t n = (size_t)L.n, m = n - 2;
+    cudaMemcpy3DParms p;
+    memset(&p, 0, sizeof p);
+    p.srcPtr = make_cudaPitchedPtr(L.r, (size_t)L.pitch * 8, n, n);
+    p.dstPtr = make_cudaPitchedPtr(uh, (size_t)L.pitch * 8, n, n);
+    p.srcPos = p.dstPos = make_cudaPos(8, 1, L.dim == 3 ? 1 : 0);
+    p.extent = make_cudaExtent(m * 8, m, L.dim == 3 ? m : 1);
+    p.kind = cudaMemcpyDeviceToDevice;
+    CK(cudaMemcpy3DAsync(&p, c->stream));
+    CK(cudaMemsetAsync(L.r, 0, (size_t)L.count * sizeof(double), c->stream));
+    TLAUNCH(c, MG_KERNEL_OTHER, 0, c->stream, DISPATCH(L, residual, L, uh, L.f, L.r, c->stream));
+  }
+  c->replay = true;
+  st = vcycle_rec(c, 1, true, c->stream);
+  c->replay = false;
+  return st;
+}
+}  // namespace mg
 
 // ---------------------------------------------------------------- ABI
 
@@ -1081,6 +1139,7 @@ static cudaError_t copy_solution_out(mg_ctx *c, double *dst, cudaStream_t s) {
     return cudaGetLastError();
   }
   double *stage = (double *)(c->dc ? c->outer.r : c->lv[0].r);
+  c->uh_in_r = false;
   const size_t cnt = (size_t)U.n * U.n * (U.dim == 3 ? U.n : 1);
   cudaError_t e = copy_pitched_to_dense(U, user_u(c), stage, s);
   if (e != cudaSuccess) return e;
@@ -1102,6 +1161,8 @@ mg_status mg_set_field(mg_ctx *c, int level, mg_field field, const double *src) 
   if (!c || !src) return fail(MG_EINVAL, "NULL argument");
   if (level < 0 || level >= c->nl) return fail(MG_EINVAL, "level %d out of range", level);
   if (field < MG_FIELD_U || field > MG_FIELD_R) return fail(MG_EINVAL, "unknown field");
+  mg_status st;
+  if ((level > 0 || field == MG_FIELD_R) && (st = mg::settle(c))) return st;
   Level &L = c->lv[level];
   void *dst = field_ptr(L, field);
   if (field == MG_FIELD_U && level == 0 && !c->dc) c->u_zero = false;
@@ -1120,6 +1181,8 @@ mg_status mg_get_field(mg_ctx *c, int level, mg_field field, double *dst) {
   if (!c || !dst) return fail(MG_EINVAL, "NULL argument");
   if (level < 0 || level >= c->nl) return fail(MG_EINVAL, "level %d out of range", level);
   if (field < MG_FIELD_U || field > MG_FIELD_R) return fail(MG_EINVAL, "unknown field");
+  mg_status st;
+  if ((level > 0 || field == MG_FIELD_R) && (st = mg::settle(c))) return st;
   Level &L = c->lv[level];
   void *src = field_ptr(L, field);
   if (L.dtype == mg::F64) {
@@ -1138,6 +1201,7 @@ mg_status mg_smooth(mg_ctx *c, int level, int sweeps) {
   if (!c) return fail(MG_EINVAL, "NULL context");
   if (level < 0 || level >= c->nl) return fail(MG_EINVAL, "level %d out of range", level);
   if (sweeps < 0) return fail(MG_EINVAL, "sweeps must be >= 0");
+  if (mg_status st = mg::settle(c)) return st;
   if (level == 0 && !c->dc) c->u_zero = false;
   return op_smooth(c, level, sweeps, c->stream);
 }
@@ -1145,24 +1209,28 @@ mg_status mg_smooth(mg_ctx *c, int level, int sweeps) {
 mg_status mg_residual(mg_ctx *c, int level) {
   if (!c) return fail(MG_EINVAL, "NULL context");
   if (level < 0 || level >= c->nl) return fail(MG_EINVAL, "level %d out of range", level);
-  return op_residual(c, level, c->stream);
+  mg_status st = mg::settle(c);
+  return st ? st : op_residual(c, level, c->stream);
 }
 
 mg_status mg_restrict(mg_ctx *c, int level) {
   if (!c) return fail(MG_EINVAL, "NULL context");
   if (level < 0 || level >= c->nl - 1) return fail(MG_EINVAL, "level %d has no coarser level", level);
-  return op_restrict(c, level, c->stream);
+  mg_status st = mg::settle(c);
+  return st ? st : op_restrict(c, level, c->stream);
 }
 
 mg_status mg_prolongate(mg_ctx *c, int level) {
   if (!c) return fail(MG_EINVAL, "NULL context");
   if (level < 0 || level >= c->nl - 1) return fail(MG_EINVAL, "level %d has no coarser level", level);
+  if (mg_status st = mg::settle(c)) return st;
   if (level == 0 && !c->dc) c->u_zero = false;
   return op_prolong(c, level, c->stream);
 }
 
 mg_status mg_coarse_solve(mg_ctx *c) {
   if (!c) return fail(MG_EINVAL, "NULL context");
+  if (mg_status st = mg::settle(c)) return st;
   if (c->nl == 1 && !c->dc) c->u_zero = false;
   return op_coarse(c, c->stream);
 }
@@ -1176,8 +1244,9 @@ mg_status mg_vcycle(mg_ctx *c) {
 mg_status mg_residual_norm(mg_ctx *c, int level, double *out) {
   if (!c || !out) return fail(MG_EINVAL, "NULL argument");
   if (level < 0 || level >= c->nl) return fail(MG_EINVAL, "level %d out of range", level);
-  mg_status st = op_norm(c, level, c->stream);
-  if (st) return st;
+  mg_status st;
+  if (level > 0 && (st = mg::settle(c))) return st;
+  if ((st = op_norm(c, level, c->stream))) return st;
   return read_norm(c, out);
 }
 

@@ -162,3 +162,70 @@ def test_complex_diffusion_residual_before_any_cycle():
     s.restrict(0)
     ref.restrict(0)
     assert np.abs(s.get_field(1, "f") - ref.get_field(1, "f")).max() <= 1e-13 * 170
+
+
+# FP64 node grids: the levels above 33 (9 in 3D), whose fields cycles of one kernel
+# per operator or the fused FP64 passes leave; red-black 2D passes form no r
+@pytest.mark.parametrize("dim,n,smoother,omega,nu,kw", [
+    (2, 65, "rbgs", 1.0, (2, 1), {}),
+    (2, 129, "rbgs", 1.0, (2, 1), {}),
+    (2, 129, "jacobi", 0.8, (1, 2), {}),
+    (2, 257, "rbgs", 1.0, (2, 2), dict(cluster_max_n=257)),
+    (2, 513, "rbgs", 1.0, (3, 2), {}),
+    (2, 513, "jacobi", 0.8, (2, 1), {}),
+    (2, 257, "jacobi", 0.8, (3, 3), dict(cluster_max_n=33)),
+    (3, 257, "rbgs", 1.0, (1, 2), {}),
+    (3, 257, "jacobi", 0.8, (2, 1), {}),
+])
+@pytest.mark.parametrize("solve", [False, True])
+def test_node_fp64(dim, n, smoother, omega, nu, kw, solve):
+    need_gpu()
+    from paper_1406_5369_gb300 import Solver
+    f, b = synth.uniform(86, (n,) * dim), synth.uniform(87, (n,) * dim)
+    u0 = synth.uniform(88, (n,) * dim)
+    kw = dict(kw, smoother=smoother, omega=0.3 if solve else omega, nu1=nu[0], nu2=nu[1], maxit=3, dirichlet=b)
+    s, ref = Solver(dim, n, **kw), Solver(dim, n, fuse=False, **kw)
+    for t in (s, ref):
+        t.set_rhs(f)
+        t.set_solution(u0)
+        if solve:
+            t.solve(0.0, raise_on_noconv=False)
+        else:
+            t.vcycle()
+    top = 33 if dim == 2 else 9
+    names = ("f", "u") if smoother == "rbgs" and dim == 2 else ("r", "f", "u")
+    order = [(l, name) for l in range(s.levels) if s.level_size(l) > top for name in names]
+    compare(s, ref, lambda l: 2.0 * dim * (n >> l) ** 2, order[::-1] + order)
+
+
+def test_node_fp64_residual_of_the_caller():
+    """Fused red-black cycles leave r as the caller's mg_residual left it."""
+    need_gpu()
+    from paper_1406_5369_gb300 import Solver
+    for n in (65, 129, 513):
+        s = Solver(2, n)
+        s.set_rhs(synth.uniform_rhs(2, n, 89))
+        s.residual(0)
+        r = s.get_field(0, "r")
+        s.vcycle()
+        s.get_field(1, "u")
+        assert np.array_equal(s.get_field(0, "r"), r)
+
+
+def test_node_fp64_batch_after_a_cycle():
+    """A context that has run a cycle of its own joins a batch with every field in place."""
+    need_gpu()
+    from paper_1406_5369_gb300 import BatchSolver, Solver
+    n = 257
+    f = synth.uniform_rhs(2, n, 90)
+    got = []
+    for own in (True, False):
+        s = Solver(2, n, smoother="jacobi", omega=0.8, nu1=2, nu2=2)
+        s.set_rhs(f)
+        s.vcycle() if own else None
+        s.set_solution(None)
+        b = BatchSolver(1)
+        b.add(s)
+        b.solve(1e-8, maxit=50)
+        got.append(s.get_solution())
+    assert np.array_equal(got[0], got[1])
