@@ -37,10 +37,12 @@ constexpr int kOut = 60;   // columns written per strip
 // Rows per chunk of a batch's problems. A warp walks its chunk alone (0.7 us a
 // row), so problems with few strips take short ones; the largest (1025^2) has a
 // chunk for each of its 512 warps. Below kBatchMinN a problem's rows are too few
-// to hide a chunk's latency (100 problems of 65^2: 3.41 ms a solve on the FP64
-// kernel, 3.49 ms here; 20 of 129^2 to 513^2: 8.51 and 8.41 ms).
-constexpr int kBatchMinN = 257;
-__host__ __device__ constexpr int batch_rows(int n) { return n <= 257 ? 8 : n <= 513 ? 16 : 40; }
+// to hide a chunk's latency, and beside smaller problems, which keep the FP64
+// kernel, it costs a launch of its own (solves of a few 33^2 to 257^2 problems:
+// 3.45 ms on the FP64 kernel, 3.53 ms with 257^2 here; 40 of them: 5.07 and 5.06;
+// four of 513^2: 6.15 and 6.04 ms).
+constexpr int kBatchMinN = 513;
+__host__ __device__ constexpr int batch_rows(int n) { return n <= 513 ? 16 : 40; }
 // A problem alone: short chunks, or too few warps; below 1025^2 the FP64 kernel's
 // one node per thread is as fast (129^2: 738 us a solve, 750 us with this one).
 constexpr int kAloneMinN = 1025;
