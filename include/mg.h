@@ -92,7 +92,14 @@ typedef struct { int kind; const double *dirichlet_values; } mg_boundary;
  * stream                : cudaStream_t for every launch, NULL = default stream
  * fuse                  : 1 = fused fine-level kernels where available,
  *                         0 = one kernel per operator (same results up to
- *                         rounding order of FMA contraction)
+ *                         rounding order of FMA contraction). Large FP64
+ *                         levels (2D from 65, 3D from 257, constant stencil)
+ *                         are then smoothed in 64-bit fixed point: each value
+ *                         to 2^-54 .. 2^-57 of the largest beside it (2D: a
+ *                         strip of 64 columns and a chunk of rows; 3D: 64 x 32
+ *                         columns and a chunk of planes), so that values far
+ *                         below that keep fewer bits than FP64 has; with 0
+ *                         they keep FP64's
  * use_graph             : 1 = replay each V-cycle from a captured CUDA graph
  * inner_cycles          : *_DC only: inner V-cycles per outer FP64 step (1..8, 0 = 1);
  *                         the first starts from e = 0, the others continue

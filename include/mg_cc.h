@@ -23,7 +23,10 @@
  *             (re-discretization)"); the coarsest grid (1, 2 or 4 cells per
  *             dimension) is solved exactly in FP64 with its inverse, formed
  *             at creation.
- * Everything runs in FP64.
+ * Fields are FP64. Large 2D levels are smoothed in 64-bit fixed point, each value
+ * to 2^-54 .. 2^-57 of the largest beside it (a strip of 64 columns, a chunk of
+ * rows); the finest level stays in FP64 arithmetic where the reaction term lets
+ * the solution decay by more than 2^-10 over such a strip and chunk.
  *
  * Conventions are those of include/mg.h: status codes (mg_status) and
  * mg_last_error() for the message; the caller owns the arena (device memory,

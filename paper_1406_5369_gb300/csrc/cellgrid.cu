@@ -704,10 +704,26 @@ mg_status read_norm(mg_cc_ctx *c, double *out) {
 // one launch per smoothing phase in place of 6 or more.
 constexpr int kFxMinN = 64;
 
+// The passes hold a strip's values as multiples of one unit, 54 to 57 bits below
+// the largest. With a reaction term the solution may decay by e^-a per cell, a =
+// sqrt(sigma / k); where that adds up to more than 2^-10 over the columns of a
+// strip and the rows of a chunk the finest level, whose values are the result,
+// stays in FP64 (its last digits would go first: sigma h^2 = 0.05, 512^2, solved to
+// the rounding floor, had relative errors of 5e-12 in place of 5e-14 where the
+// solution had fallen to 4e-12). A chunk is 8 rows or n^2 / 52 / 2432: one wave of
+// warps, 52 columns each.
+bool decays(const mg_cc_ctx *c, const Lev &L) {
+  const double ih2 = (double)L.n * (double)L.n;
+  const double rows = fmax(8.0, ih2 / (52.0 * 2432.0));
+  const double a = mg::fx2::kCols * sqrt(c->p.sigma / (c->p.c[0] * ih2)) + rows * sqrt(c->p.sigma / (c->p.c[1] * ih2));
+  return a > 10.0 * M_LN2;
+}
+
 // Level l's pass constants; false: the level keeps the kernels above.
 bool fx_args(const mg_cc_ctx *c, int l, bool corr, mg::fx2::Args &a) {
   const Lev &L = c->lv[l];
   if (c->p.dim != 2 || L.n < kFxMinN || l + 1 >= c->nl || c->p.nu1 < 1 || c->p.nu2 < 1) return false;
+  if (l == 0 && decays(c, L)) return false;
   memset(&a, 0, sizeof a);
   const double ih2 = (double)L.n * (double)L.n;
   return mg::fx2::set_operator(a, c->p.c[0] * ih2, c->p.c[1] * ih2, c->p.sigma, c->p.bc == MG_CC_NEUMANN ? 1 : 3,
