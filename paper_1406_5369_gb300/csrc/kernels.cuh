@@ -81,7 +81,7 @@ template <typename C> struct Sten {
   C c0, c1, c2;              // constant coefficients
   C inv_h2;
   C diag;                    // constant stencil: 2 (c0+c1[+c2]) / h^2
-  C rdiag;                   // 1 / diag (a division per node costs more than the stencil in FP64)
+  C rdiag;                   // 1 / diag (a division per node costs more than the stencil in FP64; FP32 divides)
 };
 
 template <typename C> __host__ Sten<C> sten_of(const Level &L) {
@@ -165,7 +165,8 @@ __global__ void k_rbgs_half(T *__restrict__ u, const T *__restrict__ f, Geo g, S
   C Au, dg;
   apply_at<DIM, VAR>(u, t.p, g, s, Au, dg);
   C u0 = ld(u + t.p);
-  st(u + t.p, VAR ? u0 + omega * (ld(f + t.p) - Au) / dg : u0 + (omega * s.rdiag) * (ld(f + t.p) - Au));
+  st(u + t.p, VAR || sizeof(C) == 4 ? u0 + omega * (ld(f + t.p) - Au) / dg
+                                    : u0 + (omega * s.rdiag) * (ld(f + t.p) - Au));
 }
 
 // omega-Jacobi: uout = uin + omega (f - A uin) / diag.
@@ -178,7 +179,8 @@ __global__ void k_jacobi(const T *__restrict__ uin, T *__restrict__ uout, const 
   C Au, dg;
   apply_at<DIM, VAR>(uin, t.p, g, s, Au, dg);
   const C u0 = ld(uin + t.p);
-  st(uout + t.p, VAR ? u0 + omega * (ld(f + t.p) - Au) / dg : u0 + (omega * s.rdiag) * (ld(f + t.p) - Au));
+  st(uout + t.p, VAR || sizeof(C) == 4 ? u0 + omega * (ld(f + t.p) - Au) / dg
+                                       : u0 + (omega * s.rdiag) * (ld(f + t.p) - Au));
 }
 
 // ---------------------------------------------------------------- residual
