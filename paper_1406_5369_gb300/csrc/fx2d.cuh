@@ -86,6 +86,8 @@ struct Args {
   Mul w[4];              // the same by boundary class (row is edge) * 2 + (column is edge)
   int edge;              // cells: weight 2u loses or gains at an edge: 1 (zero flux) or 3 (fixed value) in place of 2
   double k;              // residual = r' k
+  double km;             // k = km 2^ke, km in [1/2, 1)
+  int ke;
   double dpx, dpy, dgamma, ds, dw[4];
 };
 
@@ -513,15 +515,17 @@ __device__ __forceinline__ bool strip(const Args &a, unsigned char *ring, int la
               const long long v = (rr[q] << sh) + l;
               sq += (unsigned long long)__mul64hi(v, v);
             }
-            // sq 2^(64 - 2 sh) units squared, a unit is 2^(E - 1022 - P)
+            // sq 2^(64 - 2 sh) units squared, a unit is 2^(E - 1022 - P); with k's power
+            // of two, since the square of r' or of k alone may leave FP64's range
             const double d = __ull2double_rn(sq);
-            const int ex = 64 - 2 * sh + 2 * (E - 1022 - P) + (__double2hiint(d) >> 20);
+            const int ex = 64 - 2 * sh + 2 * (E - 1022 - P + a.ke) + (__double2hiint(d) >> 20);
             if (sq) acc += ex <= 0 ? 0.0
                            : ex >= 2047 ? __hiloint2double(0x7ff00000, 0)
                                         : __hiloint2double((ex << 20) | (__double2hiint(d) & 0xfffff),
                                                            __double2loint(d));
           } else {
-            acc += rr[0] * rr[0] + rr[1] * rr[1];
+            const double v0 = rr[0] * a.k, v1 = rr[1] * a.k;
+            acc += v0 * v0 + v1 * v1;
           }
         }
       }
@@ -614,7 +618,7 @@ __global__ void __launch_bounds__(32 * kWarps, kBlocks) k_fx2d(const __grid_cons
   if constexpr (OUT == kNorm) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if (lane == 0) a.partials[gw] = acc * (a.k * a.k);
+    if (lane == 0) a.partials[gw] = good ? acc * (a.km * a.km) : acc;
   }
 }
 
@@ -650,6 +654,8 @@ inline bool set_operator(Args &a, double kx, double ky, double sigma, int edge, 
   a.has_gamma = a.dgamma != 0.0;
   int ke;
   const double km = frexp(a.k, &ke);  // k = km 2^ke
+  a.km = km;
+  a.ke = ke;
   a.fexp = 0;
   a.fscale = 1.0;
   if (km == 0.5 && ke - 1 >= -40 && ke - 1 <= 40) {

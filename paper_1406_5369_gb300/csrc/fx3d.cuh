@@ -69,6 +69,8 @@ struct Args {
   int has_p[3], has_gamma;
   Mul p[3], gamma, w;
   double k, dp[3], dgamma, dw;
+  double km;  // k = km 2^ke
+  int ke;
 };
 
 // fx2::stored on the integer pipe, 13 instructions: the warps of a block run in
@@ -530,7 +532,7 @@ __device__ __forceinline__ bool column(const Args &a, unsigned char *smem, doubl
                 sq += (unsigned long long)__mul64hi(v, v);
               }
             const double d = __ull2double_rn(sq);
-            const int ex = 64 - 2 * sh + 2 * (E - 1022 - P) + (__double2hiint(d) >> 20);
+            const int ex = 64 - 2 * sh + 2 * (E - 1022 - P + a.ke) + (__double2hiint(d) >> 20);
             if (sq) acc += ex <= 0 ? 0.0
                            : ex >= 2047 ? __hiloint2double(0x7ff00000, 0)
                                         : __hiloint2double((ex << 20) | (__double2hiint(d) & 0xfffff),
@@ -539,7 +541,10 @@ __device__ __forceinline__ bool column(const Args &a, unsigned char *smem, doubl
 #pragma unroll
             for (int r = 0; r < 2; r++)
 #pragma unroll
-              for (int q = 0; q < 2; q++) acc += R[r][q] * R[r][q];
+              for (int q = 0; q < 2; q++) {
+                const double v = R[r][q] * a.k;
+                acc += v * v;
+              }
           }
         }
       }
@@ -621,8 +626,8 @@ template <bool JAC, int KIND, bool ZERO, bool CORR, int OUT>
 __global__ void __launch_bounds__(kThreads, 1) k_fx3d(const __grid_constant__ Args a) {
   extern __shared__ __align__(16) unsigned char smem[];
   double acc;
-  if (!column<Fix, JAC, KIND, ZERO, CORR, OUT>(a, smem, acc))
-    column<F64, JAC, kGen, ZERO, CORR, OUT>(a, smem, acc);
+  const bool good = column<Fix, JAC, KIND, ZERO, CORR, OUT>(a, smem, acc);
+  if (!good) column<F64, JAC, kGen, ZERO, CORR, OUT>(a, smem, acc);
   if constexpr (OUT == kNorm) {
     double *part = (double *)smem;
 #pragma unroll
@@ -632,7 +637,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_fx3d(const __grid_constant__ Ar
     if (threadIdx.x == 0) {
       double t = 0.0;
       for (int i = 0; i < kWarps; i++) t += part[i];
-      a.partials[(long long)blockIdx.y * gridDim.x + blockIdx.x] = t * (a.k * a.k);
+      a.partials[(long long)blockIdx.y * gridDim.x + blockIdx.x] = good ? t * (a.km * a.km) : t;
     }
   }
 }
@@ -654,6 +659,8 @@ inline bool set_operator(Args &a, const double (&k)[3], double omega, bool corr,
   a.gamma = fraction(fabs(a.dgamma), 1.0);
   int ke;
   const double km = frexp(a.k, &ke);
+  a.km = km;
+  a.ke = ke;
   a.fexp = 0;
   a.fscale = 1.0;
   if (km == 0.5 && ke - 1 >= -40 && ke - 1 <= 40) {

@@ -56,6 +56,7 @@ size_t fill(const Small2D &d, int nctas, sm2::Args &a) {
   a.nd = nd;
   a.nl = d.nlev - nd;
   const double k = d.kx > d.ky ? d.kx : d.ky;
+  if (!(k > 1e-200 && k < 1e200)) return 0;  // 1 / k is used; the general kernels take the others
   a.px = d.kx / k;
   a.py = d.ky / k;
   a.gamma = 1.0 - d.omega;
@@ -69,7 +70,7 @@ size_t fill(const Small2D &d, int nctas, sm2::Args &a) {
   a.u_top = d.u;
   a.pitch_top = d.pitch;
   a.kinv = 1.0 / k;
-  a.k2 = k * k;
+  a.k = k;
   a.norm_out = d.norm_out;
   a.uh = d.uh;
   a.fc = d.fc;

@@ -76,7 +76,7 @@ struct Args {
   double dense_k;       // coarsest k: the inverse acts on f = f' k
   double one;           // one node: u = f' one
   double *norm_out;     // norm of the top residual and its square (NULL: none)
-  double k2;            // top k squared
+  double k;             // top k
   double *uh, *fc;      // the top level's pre-smoothed u, the next level's right-hand side (NULL: not stored)
   int pitchc;
   double kc;            // k of the next level
@@ -351,7 +351,7 @@ template <bool CELL> __global__ void __launch_bounds__(kThreads, 1) k_small2d(co
       if (i > x.m) continue;
       a.u_top[(long long)(x.b0 + jl - off) * a.pitch_top + i - off] = x.U[(jl + 1) * x.pitch + i];
       if (a.norm_out) {
-        const double v = resid<CELL>(a, a.lv[0], x, jl, i);
+        const double v = resid<CELL>(a, a.lv[0], x, jl, i) * a.k;
         acc += v * v;
       }
     }
@@ -372,8 +372,8 @@ template <bool CELL> __global__ void __launch_bounds__(kThreads, 1) k_small2d(co
   if (a.norm_out && r == 0 && threadIdx.x == 0) {
     double t = 0.0;
     for (int b = 0; b < a.nctas; b++) t += sums[b];
-    a.norm_out[0] = sqrt(t * a.k2);
-    a.norm_out[1] = t * a.k2;
+    a.norm_out[0] = sqrt(t);
+    a.norm_out[1] = t;
   }
 }
 
