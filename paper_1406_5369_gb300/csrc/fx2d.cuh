@@ -47,6 +47,7 @@
 
 #include "fused2d.cuh"
 #include "mg_internal.h"
+#include "perdevice.h"
 
 namespace mg {
 namespace fx2 {
@@ -709,17 +710,18 @@ template <bool CELL, bool JAC, int KIND, int NU, bool ZERO, bool CORR, int OUT>
 cudaError_t launch(Args a, int rows, int *nparts, cudaStream_t s) {
   auto kernel = k_fx2d<CELL, JAC, KIND, NU, ZERO, CORR, OUT>;
   constexpr int smem = kWarps * kRing * 32 * (kVec * 8 * (ZERO ? 1 : 2) + (CORR ? 8 : 0));
-  // warps of one wave, found once (a race between threads finds the same)
-  static long long wave = 0;
-  if (!wave) {
+  // warps of one wave (or minus an error)
+  static PerDevice waves;
+  const long long wave = per_device(waves, [&]() -> long long {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) return -(long long)e;
     int dev = 0, sms = 0, blocks = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, 32 * kWarps, smem);
-    wave = (long long)(sms > 0 ? sms : 1) * (blocks > 0 ? blocks : 1) * kWarps;
-  }
+    return (long long)(sms > 0 ? sms : 1) * (blocks > 0 ? blocks : 1) * kWarps;
+  });
+  if (wave < 0) return (cudaError_t)-wave;
   a.nstrips = (a.n + kOut - 1) / kOut;
   a.R = rows > 0 ? (rows + 7) / 8 * 8 : chunk_rows(a.n, a.nstrips, wave);
   if (OUT == kNorm)  // one partial sum per warp

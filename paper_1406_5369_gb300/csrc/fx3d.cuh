@@ -688,15 +688,16 @@ cudaError_t launch(Args a, int *nparts, cudaStream_t s) {
   auto kernel = k_fx3d<JAC, KIND, ZERO, CORR, OUT>;
   constexpr int S = JAC ? 1 : 2, kNeed = S + (OUT != kNone) + (OUT == kRestrict) + (CORR);
   constexpr int kHalo = (kNeed + 1) / 2 * 2;
-  static int sms = 0;  // found once (a race between threads finds the same)
-  if (!sms) {
+  static PerDevice counts;  // SMs (or minus an error)
+  const long long sms = per_device(counts, [&]() -> long long {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) return -(long long)e;
     int dev = 0, v = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    sms = v > 0 ? v : 1;
-  }
+    return v > 0 ? v : 1;
+  });
+  if (sms < 0) return (cudaError_t)-sms;
   const int ox = kCols - 2 * kHalo, oy = kRows - 2 * kHalo;
   a.ntx = (a.n + ox - 1) / ox;
   a.nty = (a.n + oy - 1) / oy;

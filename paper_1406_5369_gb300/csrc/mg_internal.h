@@ -221,8 +221,8 @@ cudaError_t coarse_cycle_batched(const void *list_dev, int count, int dim, bool 
 // FP64 V-cycle of the small 2D levels on one thread-block cluster
 // (small2d.cuh): node-based or cell-centred constant-stencil grids, either
 // smoother. The top level has 2^lg cells per dimension, nlev levels down to
-// the coarsest. small2d_probe asks the device once whether the cluster fits
-// (outside any stream capture); small2d_ok answers no until it has run.
+// the coarsest. small2d_probe asks the current device once whether the cluster fits
+// (outside any stream capture); small2d_ok answers no until it has run there.
 struct Small2D {
   bool cell;
   int lg, nlev;

@@ -3,13 +3,19 @@
 
 #include <string.h>
 
+#include "perdevice.h"
+
 namespace mg {
 
 namespace {
 
-// Blocks per cluster the device places with the most shared memory a block
-// can have (16, a non-portable size, or 8); 0 = neither, -1 = not asked yet.
-int g_nctas = -1;
+// One more than the blocks per cluster the device places with the most shared
+// memory a block can have (16, a non-portable size, 8, or none).
+PerDevice g_nctas;
+int nctas() {
+  // asked by small2d_probe only: not inside a stream capture
+  return (int)per_device(g_nctas, [] { return 0LL; }) - 1;
+}
 
 template <bool CELL> void config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at, size_t smem, int nctas, cudaStream_t s) {
   memset(&cfg, 0, sizeof cfg);
@@ -136,20 +142,23 @@ template <bool CELL> cudaError_t launch(const sm2::Args &a, size_t smem, cudaStr
 }  // namespace
 
 void small2d_probe() {
-  if (g_nctas >= 0) return;
-  const int node = probe<false>(), cell = probe<true>();
-  cudaGetLastError();  // a refused query leaves no sticky error behind
-  g_nctas = node < cell ? node : cell;
+  per_device(g_nctas, [] {
+    const int node = probe<false>(), cell = probe<true>();
+    cudaGetLastError();  // a refused query leaves no sticky error behind
+    return 1LL + (node < cell ? node : cell);
+  });
 }
 
 bool small2d_ok(const Small2D &d) {
   sm2::Args a;
-  return g_nctas > 0 && fill(d, g_nctas, a) != 0;
+  const int n = nctas();
+  return n > 0 && fill(d, n, a) != 0;
 }
 
 cudaError_t small2d_cycle(const Small2D &d, cudaStream_t s) {
   sm2::Args a;
-  const size_t smem = g_nctas > 0 ? fill(d, g_nctas, a) : 0;
+  const int n = nctas();
+  const size_t smem = n > 0 ? fill(d, n, a) : 0;
   if (!smem) return cudaErrorInvalidValue;
   return d.cell ? launch<true>(a, smem, s) : launch<false>(a, smem, s);
 }
