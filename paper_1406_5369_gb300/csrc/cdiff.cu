@@ -237,45 +237,41 @@ __device__ __forceinline__ double2 face_diff(const double2 *__restrict__ u, cons
   return s;
 }
 
-// f - A u, A u = u + s e^{i theta} sum_f w_f (u - u_q) rounded as k_residual rounds
-// it (a sweep near the floor and the norm see the same residual).
-__device__ __forceinline__ double2 face_residual(const double2 *__restrict__ u, const double2 *__restrict__ f,
-                                                 const double2 *__restrict__ w, long long p, int i, int j, const Geo &g,
-                                                 Ph ph) {
-  return csub(f[p], cfma(make_double2(ph.x, ph.y), face_diff(u, w, p, i, j, g), u[p]));
-}
-
-// The difference form u + q (inv (f - A u)), inv = 1 / (s e^{i theta}), for the
-// finest level of cycles near the rounding floor (mg::near_floor): 32 FP64
-// instructions per cell. It rounds the solution once; the sum of neighbours
-// rounds values of its size several times, and a solve that went on with it came
-// to rest at 3.1 to 3.8 times the residual. Not in every cycle: with it in the
-// last sweep alone a step of 2048^2, Jacobi V(2,2), took 11.29 ms, without 10.37.
+// The difference form, inv = 1 / (s e^{i theta}):
+//   u' = u + q (inv (f - u) - sum_f w_f (u - u_q)),
+// 28 FP64 instructions per cell, for the finest level of cycles that may be near
+// the rounding floor. It rounds the solution once (the product first, then one
+// addition per part); the sum of neighbours rounds values of its size several
+// times, and a solve that went on with it came to rest at 3.1 to 3.8 times the
+// residual. With it in every cycle's last sweep a step of 2048^2, Jacobi V(2,2),
+// took 11.29 ms, without 10.37: solves take it when near_floor says so, then in
+// all post-smoothing sweeps; a cycle called by itself, in its last one.
 __device__ __forceinline__ double2 polished(const double2 *__restrict__ u, const double2 *__restrict__ f,
                                             const double2 *__restrict__ q, const double2 *__restrict__ w, long long p,
-                                            int i, int j, const Geo &g, Ph ph, Ph inv) {
-  return cadd(u[p], cmul(q[p], cmul(make_double2(inv.x, inv.y), face_residual(u, f, w, p, i, j, g, ph))));
+                                            int i, int j, const Geo &g, Ph inv) {
+  const double2 a = u[p], s = face_diff(u, w, p, i, j, g);
+  return cadd(a, cmul(q[p], cfma(make_double2(inv.x, inv.y), csub(f[p], a), make_double2(-s.x, -s.y))));
 }
 
 __global__ void __launch_bounds__(kBX * kBY) kr_jacobi_polish(const double2 *__restrict__ uin, double2 *__restrict__ uout,
                                                               const double2 *__restrict__ f,
                                                               const double2 *__restrict__ q,
-                                                              const double2 *__restrict__ w, Geo g, Ph ph, Ph inv) {
+                                                              const double2 *__restrict__ w, Geo g, Ph inv) {
   int i, j;
   if (!cell(g.n, i, j)) return;
   const long long p = (long long)j * g.sy + i;
-  uout[p] = polished(uin, f, q, w, p, i, j, g, ph, inv);
+  uout[p] = polished(uin, f, q, w, p, i, j, g, inv);
 }
 
 __global__ void __launch_bounds__(kBX * kBY) kr_rbgs_half_polish(double2 *u, const double2 *__restrict__ f,
                                                                  const double2 *__restrict__ q,
-                                                                 const double2 *__restrict__ w, Geo g, Ph ph, Ph inv,
+                                                                 const double2 *__restrict__ w, Geo g, Ph inv,
                                                                  int color) {
   const int j = blockIdx.y * kBY + threadIdx.y;
   const int i = 2 * (blockIdx.x * kBX + threadIdx.x) + ((color + j) & 1);
   if (i >= g.n || j >= g.n) return;
   const long long p = (long long)j * g.sy + i;
-  u[p] = polished(u, f, q, w, p, i, j, g, ph, inv);
+  u[p] = polished(u, f, q, w, p, i, j, g, inv);
 }
 
 __global__ void __launch_bounds__(kBX * kBY) kr_jacobi(const double2 *__restrict__ uin, double2 *__restrict__ uout,
@@ -418,7 +414,7 @@ __global__ void __launch_bounds__(kThreads) kr_norm_partials(const double2 *__re
   for (int j = blockIdx.x; j < g.n; j += gridDim.x)
     for (int i = threadIdx.x; i < g.n; i += blockDim.x) {
       const long long p = (long long)j * g.sy + i;
-      const double2 r = face_residual(u, f, w, p, i, j, g, ph);
+      const double2 r = cfma(make_double2(-ph.x, -ph.y), face_diff(u, w, p, i, j, g), csub(f[p], u[p]));
       acc = fma(r.x, r.x, fma(r.y, r.y, acc));
     }
   acc = block_sum(acc);
@@ -452,7 +448,7 @@ struct mg_cd_ctx {
   // A phased cycle has run: its finest pre-smoothed u is in level 0's wd, which
   // these cycles do not need, and r is still to be formed (to_complex).
   bool unsettled;
-  bool polish;  // this cycle's finest level ends with sweeps in difference form
+  int polish;  // sweeps in difference form that this cycle's finest level ends with: 0, 1, or 2 for a phase's all
   mg::StepGraphs graphs;
 };
 
@@ -608,24 +604,24 @@ dim3 tiles(int nx, int ny) { return dim3((unsigned)((nx + kBX - 1) / kBX), (unsi
   } while (0)
 
 // Sweeps of level l with phased faces; skip: the first sweep (Jacobi) or red
-// half-sweep is already in u; polish: in difference form.
-mg_status phased_smooth(mg_cd_ctx *c, int l, int sweeps, bool skip, bool polish) {
+// half-sweep is already in u; polish: none, the last or all of them in difference form.
+mg_status phased_smooth(mg_cd_ctx *c, int l, int sweeps, bool skip, int polish) {
+  const int fast = polish == 0 ? sweeps : polish == 1 ? sweeps - 1 : 0;
   Lev &L = c->lv[l];
   const Geo g = geo_of(L);
   const double gamma = 1.0 - c->p.omega;
   const double s = s_of(c, L);
-  const Ph ph = phase_of(c, L);
   const Ph inv = {cos(c->p.theta) / s, -sin(c->p.theta) / s};
   if (c->p.smoother == MG_RBGS) {
     for (int h = skip ? 1 : 0; h < 2 * sweeps; h++)
-      if (polish)
-        LAUNCH2(kr_rbgs_half_polish, (L.n + 1) / 2, L.n, L.u[L.cur], L.f, L.gy, L.gx, g, ph, inv, h & 1);
+      if (h >= 2 * fast)
+        LAUNCH2(kr_rbgs_half_polish, (L.n + 1) / 2, L.n, L.u[L.cur], L.f, L.gy, L.gx, g, inv, h & 1);
       else
         LAUNCH2(kr_rbgs_half, (L.n + 1) / 2, L.n, L.u[L.cur], L.gf, L.gy, L.gx, g, gamma, h & 1);
   } else {
     for (int h = skip ? 1 : 0; h < sweeps; h++) {
-      if (polish)
-        LAUNCH2(kr_jacobi_polish, L.n, L.n, L.u[L.cur], L.u[L.cur ^ 1], L.f, L.gy, L.gx, g, ph, inv);
+      if (h >= fast)
+        LAUNCH2(kr_jacobi_polish, L.n, L.n, L.u[L.cur], L.u[L.cur ^ 1], L.f, L.gy, L.gx, g, inv);
       else
         LAUNCH2(kr_jacobi, L.n, L.n, L.u[L.cur], L.u[L.cur ^ 1], L.gf, L.gy, L.gx, g, gamma);
       L.cur ^= 1;
@@ -639,12 +635,12 @@ mg_status phased_cycle(mg_cd_ctx *c, int l, bool begun) {
   mg_status st;
   if (l == c->nl - 1) return op_coarse(c);
   Lev &L = c->lv[l], &C = c->lv[l + 1];
-  if ((st = phased_smooth(c, l, c->p.nu1, begun && c->p.nu1 > 0, c->polish && l == 0 && c->p.nu2 == 0))) return st;
+  if ((st = phased_smooth(c, l, c->p.nu1, begun && c->p.nu1 > 0, l == 0 && c->p.nu2 == 0 ? c->polish : 0))) return st;
   LAUNCH2(kr_restrict, C.n, C.n, L.u[L.cur], L.f, L.gx, geo_of(L), phase_of(c, L), C.f, C.gf, C.u[C.cur], C.wd,
           geo_of(C), c->p.nu1 == 0 ? 0 : c->p.smoother == MG_RBGS ? 2 : 1, l == 0 ? L.wd : nullptr);
   if ((st = phased_cycle(c, l + 1, true))) return st;
   if ((st = op_prolong(c, l))) return st;
-  return phased_smooth(c, l, c->p.nu2, false, c->polish && l == 0);
+  return phased_smooth(c, l, c->p.nu2, false, l == 0 ? c->polish : 0);
 }
 
 mg_status vcycle_rec(mg_cd_ctx *c, int l) {
@@ -888,7 +884,7 @@ mg_status mg_cd_coarse_solve(mg_cd_ctx *c) {
 
 mg_status mg_cd_vcycle(mg_cd_ctx *c) {
   if (!c) return cdfail(MG_EINVAL, "NULL context");
-  c->polish = true;  // how near the floor this cycle is, is not known here
+  c->polish = 1;  // how near the floor this cycle is, is not known here
   c->unsettled = c->phased && c->nl > 1;
   return vcycle_rec(c, 0);
 }
@@ -912,7 +908,7 @@ mg_status mg_cd_solve(mg_cd_ctx *c, double tol, int *iters, double *relres, doub
   int k = 0;
   double rho = r0 > 0.0 ? 1.0 : 0.0, last = INFINITY;
   while (r0 > 0.0 && rho > tol && k < c->p.maxit) {
-    c->polish = mg::near_floor(rho, last);
+    c->polish = mg::near_floor(rho, last) ? 2 : 0;
     if ((st = solve_step(c, k))) return st;
     double rk;
     if ((st = read_norm(c, &rk))) return st;

@@ -225,11 +225,12 @@ __device__ __forceinline__ double neighbours(const double *__restrict__ u, doubl
 }
 
 // POLISH: the difference form u + wd (f - A u), for the finest level of cycles
-// near the rounding floor (mg::near_floor). It rounds the solution once; the sum
-// of neighbours rounds values of the size of diag u several times, and a solve
-// that went on with it came to rest at 2 to 2.7 times the residual (3D, 8^3 to
-// 128^3). Not in every cycle: with it in the last sweep alone a solve of 128^3,
-// V(2,2), took 3.59 ms, without 3.33.
+// that may be near the rounding floor. It rounds the solution once; the sum of
+// neighbours rounds values of the size of diag u several times, and a solve that
+// went on with it came to rest at 2 to 2.7 times the residual (3D, 8^3 to 128^3).
+// With it in every cycle's last sweep a solve of 128^3, V(2,2), took 3.59 ms,
+// without 3.33: solves take it when near_floor says so, then in all
+// post-smoothing sweeps; a cycle called by itself, in its last one.
 template <int DIM, bool POLISH>
 __global__ void __launch_bounds__(kBX * kBY) kv_rbgs_half(double *u, const double *__restrict__ f, Geo g, Coef s,
                                                           double gamma, int color) {
@@ -512,7 +513,7 @@ struct mg_cc_ctx {
   double *partials;  // kNormBlocks norm partial sums
   double *norm_out;  // the norm (and its square)
   cudaStream_t s;
-  bool polish;       // this cycle's finest level ends with sweeps in difference form
+  int polish;        // sweeps in difference form that this cycle's finest level ends with: 0, 1, or 2 for a phase's all
   // The fields that a V-cycle leaves besides level 0's u (r of level 0; u, f and r
   // of the others) are formed when a call needs them (settle): the cycle keeps the
   // finest level's pre-smoothed u in its r, and the next level's f.
@@ -811,8 +812,9 @@ mg_status vcycle_rec(mg_cc_ctx *c, int l, bool zero = false, int *nparts = nullp
   } while (0)
 
 // Sweeps of level l; begun: the first sweep (Jacobi) or red half-sweep is in u;
-// polish: in difference form.
-mg_status general_smooth(mg_cc_ctx *c, int l, int sweeps, bool begun, bool polish) {
+// polish: none, the last or all of them in difference form.
+mg_status general_smooth(mg_cc_ctx *c, int l, int sweeps, bool begun, int polish) {
+  const int fast = polish == 0 ? sweeps : polish == 1 ? sweeps - 1 : 0;
   Lev &L = c->lv[l];
   const Geo g = geo_of(L);
   const Coef s = coef_of(c, L);
@@ -820,10 +822,10 @@ mg_status general_smooth(mg_cc_ctx *c, int l, int sweeps, bool begun, bool polis
   const dim3 block(kBX, kBY);
   if (c->p.smoother == MG_RBGS) {
     for (int h = begun ? 1 : 0; h < 2 * sweeps; h++)
-      DIMCALL2(c->p.dim, polish, kv_rbgs_half, tiles(c, (L.n + 1) / 2, L.n), block, L.u[L.cur], L.f, g, s, gamma, h & 1);
+      DIMCALL2(c->p.dim, h >= 2 * fast, kv_rbgs_half, tiles(c, (L.n + 1) / 2, L.n), block, L.u[L.cur], L.f, g, s, gamma, h & 1);
   } else {
     for (int h = begun ? 1 : 0; h < sweeps; h++) {
-      DIMCALL2(c->p.dim, polish, kv_jacobi, tiles(c, L.n, L.n), block, L.u[L.cur], L.u[L.cur ^ 1], L.f, g, s, gamma);
+      DIMCALL2(c->p.dim, h >= fast, kv_jacobi, tiles(c, L.n, L.n), block, L.u[L.cur], L.u[L.cur ^ 1], L.f, g, s, gamma);
       L.cur ^= 1;
     }
   }
@@ -863,7 +865,7 @@ mg_status general_cycle(mg_cc_ctx *c, int l, int start) {
     return MG_OK;
   }
   if (start == 0) CCK(cudaMemsetAsync(L.u[L.cur], 0, (size_t)L.count * sizeof(double), c->s));
-  if ((st = general_smooth(c, l, c->p.nu1, start == 1 && c->p.nu1 > 0, c->polish && l == 0 && c->p.nu2 == 0))) return st;
+  if ((st = general_smooth(c, l, c->p.nu1, start == 1 && c->p.nu1 > 0, l == 0 && c->p.nu2 == 0 ? c->polish : 0))) return st;
   // the next level: u from its first sweep unless it solves, or starts by itself
   const bool last = l + 2 == c->nl, own = !last && (small_desc(c, l + 1, true).lg > 0 || level_fx(c, l + 1));
   const int first = last || own || c->p.nu1 == 0 ? 0 : c->p.smoother == MG_RBGS ? 2 : 1;
@@ -873,7 +875,7 @@ mg_status general_cycle(mg_cc_ctx *c, int l, int start) {
   else if (own) st = vcycle_rec(c, l + 1, true);
   else st = general_cycle(c, l + 1, 1);
   if (st || (st = op_prolong(c, l))) return st;
-  return general_smooth(c, l, c->p.nu2, false, c->polish && l == 0);
+  return general_smooth(c, l, c->p.nu2, false, l == 0 ? c->polish : 0);
 }
 
 // Algorithm 1 from level l down; coarse levels start from zero (`zero`: u_l
@@ -1121,7 +1123,7 @@ mg_status mg_cc_coarse_solve(mg_cc_ctx *c) {
 
 mg_status mg_cc_vcycle(mg_cc_ctx *c) {
   if (!c) return ccfail(MG_EINVAL, "NULL context");
-  c->polish = polishes(c);  // how near the floor this cycle is, is not known here
+  c->polish = polishes(c) ? 1 : 0;  // how near the floor this cycle is, is not known here
   c->unsettled = c->nl > 1;
   return vcycle_rec(c, 0);
 }
@@ -1146,7 +1148,7 @@ mg_status mg_cc_solve(mg_cc_ctx *c, double tol, int *iters, double *relres, doub
   int k = 0;
   double rho = r0 > 0.0 ? 1.0 : 0.0, last = INFINITY;
   while (r0 > 0.0 && rho > tol && k < c->p.maxit) {
-    c->polish = polishes(c) && mg::near_floor(rho, last);
+    c->polish = polishes(c) && mg::near_floor(rho, last) ? 2 : 0;
     if ((st = solve_step(c, k))) return st;
     double rk;
     if ((st = read_norm(c, &rk))) return st;
