@@ -874,7 +874,7 @@ def run_c4(args):
     names = {"pre": "fused variable-stencil pre-smoothing + residual + restriction list launches (k_pre2d<float,2,Z,VAR>)",
              "post": "fused variable-stencil interpolation + post-smoothing list launches (k_post2d<float,1,VAR>)",
              "coarse": "single-block coarse cycles, one block per problem (latency-bound, time only)",
-             "outer": "FP64 outer residual with FP64 harmonic faces (kb_dc_residual<2,float,VAR>; FP64-issue bound)",
+             "outer": "FP64 outer residual with FP64 harmonic faces (kb_dc_residual_var2d<float> from 513^2 on, kb_dc_residual<2,float,VAR> below; FP64 pipe and integer issue)",
              "update": "FP64 outer update u += e (kb_dc_update)"}
     klines = []
     for k, (ms_k, n_k, by_k) in kinds.items():

@@ -20,9 +20,9 @@
 // reached is the same. Chunks with non-finite or out-of-range values, and
 // coefficients that are negative or not finite, are done in FP64.
 //
-// Bound: the FP64 pipe (60 %) and the integer ALU (53 %) together. 36 problems
-// of 33^2 to 1025^2 (8.4 M nodes): 120 us; 313 MB, 47 us of HBM. The FP64 kernel
-// took 4.9 ms for 1021 problems of the same mix, 174 us in proportion.
+// Bound: the FP64 pipe (57 %) and the integer ALU (54 %) together. 12 problems of
+// 513^2 and 1025^2 (7.9 M nodes): 95 us; 290 MB, 43 us of HBM. The FP64 kernel took
+// 4.9 ms for 1021 problems of 33^2 to 1025^2, 174 us for 8.4 M nodes in proportion.
 #pragma once
 
 #include "fx2d.cuh"

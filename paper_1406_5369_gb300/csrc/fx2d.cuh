@@ -14,10 +14,10 @@
 //   When a row with a larger exponent arrives the window is shifted right
 //   (warp-uniform, rare). P (54 .. 57) is chosen on the host from a bound on
 //   the growth of the values over the sweeps and on the residual
-//   (fx2d_node.cu: headroom), so no sum below can overflow, whatever the
-//   data. u loses nothing within a factor 2^(P - 53) of the largest value
-//   and is cut at 2^-P of it otherwise, a quarter to a sixteenth of an FP64
-//   unit in its last place. f' carries 22 more bits (FL), used by the
+//   (set_operator), so no sum below can overflow, whatever the data. u loses
+//   nothing within a factor 2^(P - 53) of the largest value and is cut at 2^-P
+//   of it otherwise, half to a sixteenth of an FP64 unit in that value's last
+//   place. f' carries 22 more bits (FL), used by the
 //   residual: h^2 f is far smaller than u, and its relative precision decides
 //   that of the solution.
 //   Sweep: u' = W (f' + px (uw + ue) + py (us + un)) + gamma u, max(px, py)
@@ -29,12 +29,14 @@
 // A strip that meets Inf or NaN, or whose exponents leave 128 .. 1900, is
 // done again in FP64 arithmetic by the same code (Arith = F64).
 //
-// Bound: integer issue (the ALU at 60 % while a warp runs; 64 columns of which
-// 52 are written and the rows before a chunk are 1.3 times the minimal work),
-// then HBM (400 MB at 6.7 TB/s: 60 us). 4097^2, V(2,2), one cycle's level in
-// us, FP64 kernels -> these: red-black omega = 1, fused FP64 passes and norm
-// 1062 -> 191 (pre), 654 + 378 -> 234 (post with the norm); Jacobi, one kernel
-// per operator, 1453 -> 235, 1294 + 398 -> 283.
+// Bound: integer issue (the ALU at 59 to 63 % while a warp runs, the FP64 pipe, on
+// which the conversions issue, at 35 to 54 % and 70 to 74 % in the passes with a
+// norm; 64 columns of which 52 are written and the rows before a chunk are 1.3
+// times the minimal work), then HBM (430 MB at 6.7 TB/s: 64 us). 4097^2, V(2,2),
+// one cycle's level in us, FP64 kernels -> these: red-black omega = 1, fused FP64
+// passes and norm 1062 -> 193 (pre), 654 + 378 -> 257 (post with the norm; 234 when
+// it was that of the unrounded values); Jacobi, one kernel per operator, 1453 ->
+// 231, 1294 + 398 -> 307 (283).
 //
 // The same pass serves node-based grids (values on boundary nodes stay, full
 // weighting, bilinear interpolation) and cell-centred ones (a missing
@@ -159,7 +161,7 @@ __device__ __forceinline__ double to_dbl(long long x, int E, int P) {
 
 // x as to_dbl stores it: rounded to 53 bits. A pass that forms the norm rounds
 // each node's last update with it, so that the norm is that of the stored
-// solution: the bits beyond FP64 would hide its rounding (4097^2, smooth data,
+// solution: the bits beyond FP64 would hide its rounding (2049^2, smooth data,
 // at the rounding floor: 0.09 of the residual of what was returned). Both
 // conversions issue on the FP64 pipe.
 __device__ __forceinline__ long long stored(long long x) { return __double2ll_rn(__ll2double_rn(x)); }

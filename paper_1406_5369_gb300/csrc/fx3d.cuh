@@ -21,11 +21,11 @@
 // registers and the published planes. A block whose data the fixed point
 // cannot hold starts again in FP64.
 //
-// Bound: integer issue (the ALU at 55 % while a block runs, 16 warps per SM) on
-// 1.5 to 2 times the nodes, since the tiles' recomputed edges count: 257^3,
+// Bound: integer issue (the ALU at 61 to 68 % while a block runs, 16 warps per SM)
+// on 1.5 to 2 times the nodes, since the tiles' recomputed edges count: 257^3,
 // V(2,2) red-black, one cycle's level in us, FP64 half-sweeps, residual,
-// restriction and norm one by one -> these: 971 -> 728 (pre), 740 + 265 -> 831
-// (post with the norm).
+// restriction and norm one by one -> these: 971 -> 717 (pre), 740 + 265 -> 841
+// (post with the norm; 831 when it was that of the unrounded values).
 #pragma once
 
 #include "fx2d.cuh"

@@ -27,7 +27,7 @@
 // whose boundary faces then only change the diagonal (weights kx, ky = edge
 // instead of 2 on u).
 //
-// Measured per V(2,1) cycle from 129^2, with the residual norm: 54 us, one
+// Measured per V(2,1) cycle from 129^2, with the residual norm: 57 us, one
 // launch, in place of 232 us in seven (block tiles for 129^2 and 65^2, the
 // single-block cycle below, the norm). About 20 us are barriers (0.5 us each),
 // the rest FP64 issue: 33^2 on all blocks instead of block 0 saved 5 us, a level
