@@ -232,7 +232,7 @@ mg_status mg_get_solution(mg_ctx *ctx, double *u);
  * the levels are the inner hierarchy (U = correction e, F = defect d).
  * A V-cycle leaves U, F and R of every level with fuse = 0. With fuse = 1 it
  * leaves no R where smoothing, residual and restriction are one kernel (2D,
- * red-black), and no coarser field below a level that one block or one cluster
+ * red-black, one or two sweeps), and no coarser field below a level that one block or one cluster
  * takes with everything under it (2D: 65 in *_DC precisions, cluster_max_n; FP64:
  * 33; 3D: 17, FP64 9). Larger FP64 levels that the cluster or the fixed-point
  * passes take do leave theirs: the first call that reads or changes R of level 0

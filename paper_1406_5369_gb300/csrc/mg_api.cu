@@ -342,7 +342,7 @@ int fused_sweeps(const mg_ctx *c, int nu) {
   return c->opt.fuse_depth > 0 && c->opt.fuse_depth < nu ? c->opt.fuse_depth : nu;
 }
 
-bool level_fused(mg_ctx *c, int l) {
+bool level_fused(const mg_ctx *c, int l) {
   if (!c->opt.fuse || c->opt.smoother != MG_RBGS || l + 1 >= c->nl) return false;
   return mg::d2::fused_ok(c->lv[l], c->lv[l + 1], fused_sweeps(c, c->opt.nu1)) &&
          mg::d2::fused_ok(c->lv[l], c->lv[l + 1], fused_sweeps(c, c->opt.nu2));
@@ -374,9 +374,10 @@ mg_status fx3_pass(mg_ctx *c, int l, int kind, void *in, void *out, bool zero, b
   return MG_OK;
 }
 
-// A cycle of one kernel per operator forms r (the fused red-black 2D passes do
-// not, and leave what is there): the pre-smoothed solution goes to r, where it stays.
-bool keeps_uh(const mg_ctx *c) { return c->dim == 3 || c->opt.smoother == MG_JACOBI; }
+// A cycle of one kernel per operator forms r (the fused red-black 2D passes, of one
+// or two sweeps, do not, and leave what is there): where the level would run so,
+// the pre-smoothed solution goes to r and stays there.
+bool keeps_uh(const mg_ctx *c) { return !level_fused(c, 0); }
 
 // The cluster V-cycle of levels l .. nl-1 (small2d.cuh); lg = 0 when the
 // context or the level does not take it. cluster_max_n sets its largest level.

@@ -229,3 +229,20 @@ def test_node_fp64_batch_after_a_cycle():
         b.solve(1e-8, maxit=50)
         got.append(s.get_solution())
     assert np.array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("n,nu", [(65, (2, 0)), (129, (3, 2)), (513, (3, 2)), (257, (1, 4))])
+def test_node_fp64_red_black_without_fused_passes(n, nu):
+    """Red-black cycles with no or more than two sweeps a phase form r on every level above 33."""
+    need_gpu()
+    from paper_1406_5369_gb300 import Solver
+    f, u0 = synth.uniform_rhs(2, n, 86), synth.uniform(88, (n, n))
+    u0[0], u0[-1], u0[:, 0], u0[:, -1] = 0, 0, 0, 0
+    kw = dict(nu1=nu[0], nu2=nu[1])
+    s, ref = Solver(2, n, **kw), Solver(2, n, fuse=False, **kw)
+    for t in (s, ref):
+        t.set_rhs(f)
+        t.set_solution(u0)
+        t.vcycle()
+    order = [(l, name) for l in range(s.levels) if s.level_size(l) > 33 for name in ("r", "f", "u")]
+    compare(s, ref, lambda l: 4.0 * (n >> l) ** 2, order)
