@@ -5,7 +5,8 @@
 //
 // A graph holds the context's buffers, which live as long as the context, and
 // is keyed by the live-buffer state it was captured in. The first two steps of
-// a context's first solve run without one: short solves never pay for capture.
+// a context's first solve run without one: short solves never pay for capture. So
+// does every step for which none can be made.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -48,30 +49,40 @@ cudaError_t step(StepGraphs &g, int k, cudaStream_t &stream, Key key, SetKey set
     *status = record();
     return cudaSuccess;
   }
-  cudaError_t e = cudaSuccess;
-  if (!g.cap && (e = cudaStreamCreateWithFlags(&g.cap, cudaStreamNonBlocking)) != cudaSuccess) return e;
+  // Another thread's capture in the global mode forbids the calls below in threads
+  // of that mode, and would be spoilt by them: not so in the thread-local mode.
+  struct Mode {
+    cudaStreamCaptureMode m = cudaStreamCaptureModeThreadLocal;
+    Mode() { cudaThreadExchangeStreamCaptureMode(&m); }
+    ~Mode() { cudaThreadExchangeStreamCaptureMode(&m); }
+  } mode;
   StepGraphs::Slot &s = g.slot[g.next];
-  g.next = (g.next + 1) & 3;
-  if (s.valid) cudaGraphExecDestroy(s.exec);
-  s.valid = false;
-  if ((e = cudaStreamBeginCapture(g.cap, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return e;
-  const cudaStream_t user = stream;
-  stream = g.cap;
-  *status = record();
-  stream = user;
-  s.post = key();
-  set_key(now);
-  cudaGraph_t graph = nullptr;
-  e = cudaStreamEndCapture(g.cap, &graph);
-  if (*status == 0 && e == cudaSuccess && (e = cudaGraphInstantiate(&s.exec, graph, 0)) == cudaSuccess) {
-    s.valid = true;
+  if ((g.cap || cudaStreamCreateWithFlags(&g.cap, cudaStreamNonBlocking) == cudaSuccess) &&
+      cudaStreamBeginCapture(g.cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+    g.next = (g.next + 1) & 3;
+    if (s.valid) cudaGraphExecDestroy(s.exec);
+    s.valid = false;
+    const cudaStream_t user = stream;
+    stream = g.cap;
+    *status = record();
+    stream = user;
+    s.post = key();
+    set_key(now);
+    cudaGraph_t graph = nullptr;
+    const cudaError_t e = cudaStreamEndCapture(g.cap, &graph);
+    s.valid = *status == 0 && e == cudaSuccess && cudaGraphInstantiate(&s.exec, graph, 0) == cudaSuccess;
     s.key = now;
+    if (graph) cudaGraphDestroy(graph);
+    if (s.valid) {
+      const cudaError_t launched = cudaGraphLaunch(s.exec, stream);
+      if (launched == cudaSuccess) set_key(s.post);
+      return launched;
+    }
   }
-  if (graph) cudaGraphDestroy(graph);
-  if (!s.valid) return e;
-  e = cudaGraphLaunch(s.exec, stream);
-  if (e == cudaSuccess) set_key(s.post);
-  return e;
+  // no graph (no memory for one, say): the step's launches themselves
+  cudaGetLastError();
+  *status = record();
+  return cudaSuccess;
 }
 
 }  // namespace mg
